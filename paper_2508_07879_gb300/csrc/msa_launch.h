@@ -285,7 +285,7 @@ cudaError_t launch_msa_learned(const LaunchParams &p, const KernelChoice &kc, di
                                size_t smem, cudaStream_t stream);
 
 // ---------------------------------------------------------------------------------------------
-// Training of the learned decoder and its helpers (nms_train.cu).
+// Training of the learned decoder (nms_train.cu); the error sampler and the logical test (evaluate.cu).
 // ---------------------------------------------------------------------------------------------
 // Recorded check-node state of one iteration: 4 words per check, word f of check i at f*m + i:
 //   0: min1 (FP32 bits)  1: min2 (FP32 bits)  2: sign bits, bit j = [q_j < 0]
@@ -331,9 +331,22 @@ cudaError_t launch_gather_grad(const float *grad_slot, const uint32_t *eslot, in
 cudaError_t launch_adam(float *param, const float *grad, float *m1, float *m2, int64_t count, int32_t step,
                         float lr, float beta1, float beta2, float eps, cudaStream_t stream);
 cudaError_t launch_sample(const DeviceGraph &g, uint64_t seed, int64_t first_shot, int32_t batch, double p_lo,
-                          double p_hi, uint8_t *err, uint8_t *syn, int grid, cudaStream_t stream);
-cudaError_t launch_logical(const uint8_t *logicals, int32_t k, int32_t n, const uint8_t *err, const uint8_t *dec,
-                           const uint8_t *ok, int32_t batch, uint8_t *fail, int grid, cudaStream_t stream);
+                          double p_hi, uint8_t *err, uint8_t *syn, int sm_count, cudaStream_t stream);
+// Shared memory of the sampler's block for a graph (its kernel may need the opt-in above 48 KB).
+const void *sample_kernel_ptr();
+size_t sample_smem(int32_t m, int32_t n);
+
+// Logical test: `shots` decoded shots per block at a time and the block's shared memory; shots = 0: a
+// code too long for the tiled kernel, tested one shot per block.
+struct LogicalPlan {
+    int shots;
+    size_t smem;
+    const void *kernel;
+};
+LogicalPlan plan_logical(int32_t k, int32_t n);
+cudaError_t launch_logical(const LogicalPlan &pl, const uint8_t *logicals, int32_t k, int32_t n, const uint8_t *err,
+                           const uint8_t *dec, const uint8_t *ok, int32_t batch, uint8_t *fail, int sm_count,
+                           cudaStream_t stream);
 
 // Shared memory of one training shot (forward: q slots, gamma, targets, syndrome; backward adds
 // the recomputed r slots and the recorded state of two iterations).  The syndrome loss adds the

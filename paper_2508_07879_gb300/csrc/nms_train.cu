@@ -480,78 +480,6 @@ __global__ void adam_kernel(float *__restrict__ param, const float *__restrict__
     }
 }
 
-// SplitMix64 (Steele, Lea and Flood, OOPSLA 2014): the output of one step from state x.
-__device__ __forceinline__ uint64_t splitmix64(uint64_t x)
-{
-    uint64_t z = x + 0x9E3779B97F4A7C15ull;
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return z ^ (z >> 31);
-}
-
-// Errors at a per-shot rate and their syndromes, one block per shot.  Counter-based keying
-// (seed, shot, qubit): u = top 53 bits of mix(mix(mix(seed) + shot) + qubit) / 2^53;
-// p_shot = p_lo + p_span * u(qubit n); e_q = [u(q) < p_shot]; s_i = XOR of e over row i.
-__global__ void sample_kernel(const DeviceGraph g, uint64_t seed, int64_t first_shot, int32_t batch, double p_lo,
-                              double p_span, uint8_t *__restrict__ err, uint8_t *__restrict__ syn)
-{
-    extern __shared__ __align__(16) unsigned char es[];
-    const int M = g.m, N = g.n, T = blockDim.x, tid = threadIdx.x;
-    const uint64_t k_seed = splitmix64(seed);
-    for (int b = blockIdx.x; b < batch; b += gridDim.x) {
-        const uint64_t k_shot = splitmix64(k_seed + uint64_t(first_shot + b));
-        const double un = double(splitmix64(k_shot + uint64_t(N)) >> 11) * 1.1102230246251565e-16;   // 2^-53
-        const double thr = __dmul_rn(__dadd_rn(p_lo, __dmul_rn(p_span, un)), 9007199254740992.0);     // p * 2^53
-        for (int q = tid; q < N; q += T) {
-            const uint8_t e = double(splitmix64(k_shot + uint64_t(q)) >> 11) < thr ? 1 : 0;
-            es[q] = e;
-            err[size_t(b) * N + q] = e;
-        }
-        __syncthreads();
-        for (int c = tid; c < M; c += T) {
-            const int deg = __ldg(g.rdeg + c);
-            uint32_t par = 0;
-            for (int j = 0; j < deg; ++j) par ^= es[__ldg(g.ecol + size_t(j) * M + c)];
-            syn[size_t(b) * M + c] = uint8_t(par);
-        }
-        __syncthreads();
-    }
-}
-
-// fail_b = !ok_b OR some logical operator l has odd overlap with the residual e_b XOR e_hat_b.
-__global__ void logical_kernel(const uint8_t *__restrict__ logicals, int32_t K, int32_t N, const uint8_t *__restrict__ err,
-                               const uint8_t *__restrict__ dec, const uint8_t *__restrict__ ok, int32_t batch,
-                               uint8_t *__restrict__ fail)
-{
-    extern __shared__ __align__(16) uint32_t lw[];
-    const int W = (N + 31) / 32, T = blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int nwarp = (T + 31) / 32;
-    uint32_t *rw = lw + size_t(K) * W;
-    for (int idx = warp; idx < K * W; idx += nwarp) {   // pack L row by row, 32 qubits per word
-        const int l = idx / W, wd = idx - l * W, q = wd * 32 + lane;
-        const uint32_t bits = __ballot_sync(0xffffffffu, q < N && logicals[size_t(l) * N + q]);
-        if (lane == 0) lw[idx] = bits;
-    }
-    for (int b = blockIdx.x; b < batch; b += gridDim.x) {
-        __syncthreads();
-        for (int wd = warp; wd < W; wd += nwarp) {
-            const int q = wd * 32 + lane;
-            const bool r = q < N && ((err[size_t(b) * N + q] ^ dec[size_t(b) * N + q]) & 1u);
-            const uint32_t bits = __ballot_sync(0xffffffffu, r);
-            if (lane == 0) rw[wd] = bits;
-        }
-        __syncthreads();
-        int odd = 0;
-        for (int l = tid; l < K; l += T) {
-            uint32_t par = 0;
-            for (int wd = 0; wd < W; ++wd) par ^= uint32_t(__popc(lw[l * W + wd] & rw[wd]));
-            odd |= int(par & 1u);
-        }
-        odd = __syncthreads_or(odd);
-        if (tid == 0) fail[b] = (ok[b] == 0 || odd) ? 1 : 0;
-    }
-}
-
 }  // namespace kern
 
 // Compiled training variants: uniform row degree 6..8 with column-degree bucket 4 or 8, else a
@@ -647,21 +575,6 @@ cudaError_t launch_adam(float *param, const float *grad, float *m1, float *m2, i
     const double bc2 = 1.0 - std::pow(double(beta2), double(step));
     kern::adam_kernel<<<elementwise_grid(count), 256, 0, stream>>>(param, grad, m1, m2, count, beta1, beta2, eps,
                                                                    float(double(lr) / bc1), float(std::sqrt(bc2)));
-    return cudaGetLastError();
-}
-
-cudaError_t launch_sample(const DeviceGraph &g, uint64_t seed, int64_t first_shot, int32_t batch, double p_lo,
-                          double p_hi, uint8_t *err, uint8_t *syn, int grid, cudaStream_t stream)
-{
-    kern::sample_kernel<<<grid, 256, size_t(g.n), stream>>>(g, seed, first_shot, batch, p_lo, p_hi - p_lo, err, syn);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_logical(const uint8_t *logicals, int32_t k, int32_t n, const uint8_t *err, const uint8_t *dec,
-                           const uint8_t *ok, int32_t batch, uint8_t *fail, int grid, cudaStream_t stream)
-{
-    const size_t smem = (size_t(k) + 1) * size_t((n + 31) / 32) * 4;
-    kern::logical_kernel<<<grid, 128, smem, stream>>>(logicals, k, n, err, dec, ok, batch, fail);
     return cudaGetLastError();
 }
 

@@ -244,8 +244,8 @@ int qldpc_sample_errors(const qldpc_graph *g, uint64_t seed, int64_t first_shot,
     if (batch == 0) return QLDPC_OK;
     if (!out_err || !out_syn) return QLDPC_ERR_INVALID_ARG;
     if (int rc = check_device(g)) return rc;
-    const int grid = int(std::min<int64_t>(batch, int64_t(g->sm_count) * 8));
-    return cuda_status(launch_sample(g->dg, seed, first_shot, batch, p_lo, p_hi, out_err, out_syn, grid,
+    if (int rc = ensure_kernel_attrs(sample_kernel_ptr(), sample_smem(g->m, g->n), g->smem_optin)) return rc;
+    return cuda_status(launch_sample(g->dg, seed, first_shot, batch, p_lo, p_hi, out_err, out_syn, g->sm_count,
                                      static_cast<cudaStream_t>(stream)));
 }
 
@@ -257,12 +257,14 @@ int qldpc_logical_failures(const uint8_t *logicals, int32_t k, int32_t n, const 
     if (batch == 0) return QLDPC_OK;
     if (!logicals || !errors || !decisions || !ok || !out_fail) return QLDPC_ERR_INVALID_ARG;
     if ((size_t(k) + 1) * size_t((n + 31) / 32) * 4 > 48 * 1024) return QLDPC_ERR_UNSUPPORTED;
-    int dev = 0, sms = 0;
+    int dev = 0, sms = 0, optin = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
         return QLDPC_ERR_CUDA;
-    const int grid = int(std::min<int64_t>(batch, int64_t(sms) * 8));
-    return cuda_status(launch_logical(logicals, k, n, errors, decisions, ok, batch, out_fail, grid,
+    const LogicalPlan pl = plan_logical(k, n);
+    if (int rc = ensure_kernel_attrs(pl.kernel, pl.smem, size_t(optin))) return rc;
+    return cuda_status(launch_logical(pl, logicals, k, n, errors, decisions, ok, batch, out_fail, sms,
                                       static_cast<cudaStream_t>(stream)));
 }
 
