@@ -21,7 +21,7 @@
 //     reads one word per check and the block settles the test with one __syncthreads_and, so an
 //     iteration costs two block barriers (the paper's kernel: four);
 //   * the check step keeps no argmin: min over S_v(m)\n is min2 where |q_n| equals min1 and min1
-//     elsewhere (min2 = min1 when the minimum is shared), which is exact.
+//     elsewhere (min2 = min1 when the minimum is shared), which is exact (FP32: other_min below).
 //
 // Arithmetic is operation-for-operation that of the CPU oracle:
 //   r = sign * (alpha * min_{j != n} |q_j|)
@@ -260,6 +260,25 @@ __device__ __forceinline__ void two_smallest_signed(const float *q, float &m1s, 
     }
 }
 
+// sign * min over the other messages, for one FP32 message q of a row with smallest magnitudes m1 <= m2:
+// min(|q|, m2) is m1 where q holds the minimum and m2 elsewhere, so the minimum over the others is the
+// one of the two that it is not, and since the bits of non-negative floats are whole numbers it is
+// bits(m1) + bits(m2) - bits(min(|q|, m2)), exactly.  The sign of q rides along (min.xorsign with m2 >= 0: its
+// bit survives the subtraction modulo 2^32) and the check's factor sits in the sum's bit 31.  Two
+// instructions where a comparison, a selection and a sign XOR took three, and one on the ALU pipe
+// (which bounds the kernels) instead of three.  A NaN q counts as not holding the minimum, as in the comparison.
+// LP-1054, 65536 shots at p = 0.05 in pairs: 3958 -> 3627 us; rows of 9 on [H | I], 8191 shots: 926 -> 849 us;
+// learned, 16384 shots: 752 -> 727 us.  (An XOR of the three bit patterns serves as well but stays on the ALU
+// pipe: 3693 us.)
+__device__ __forceinline__ uint32_t other_sum(float m1, float m2, uint32_t factor_bit31)
+{
+    return __float_as_uint(m1) + __float_as_uint(m2) + factor_bit31;
+}
+__device__ __forceinline__ float other_min(float q, float m2, uint32_t sum)
+{
+    return __uint_as_float(sum - __float_as_uint(min_xorsign_abs(q, m2)));
+}
+
 // The check update's reductions of one row: its two smallest magnitudes m1 <= m2 (with multiplicity)
 // and the parity of its messages' sign bits (bit 31 of sx).  FP32 rows of exact degree take the parity
 // with the smallest magnitude (one instruction per pair of messages fewer); the others xor the signs.
@@ -280,6 +299,31 @@ __device__ __forceinline__ void row_minima(const typename P::acc_t *q, int deg, 
         two_smallest<P, DC, UNIFORM>(q, deg, m1, m2);
     }
 }
+
+// r of each message of a row from its two smallest magnitudes and negall = [(-1)^{s_m} prod of all signs < 0].
+// FP32 forms it from other_min; the fixed-point forms scale the two magnitudes first (a floor each).
+template <class P>
+struct RowOut {
+    typename P::mag_t m1, r1, r2;
+    __device__ __forceinline__ RowOut(typename P::mag_t a1, typename P::mag_t a2, uint32_t negall, const LaunchParams &p)
+        : m1(a1), r1(P::presign(P::scale(a1, p), negall)), r2(P::presign(P::scale(a2, p), negall)) {}
+    __device__ __forceinline__ typename P::acc_t operator()(typename P::acc_t q, const LaunchParams &) const
+    {
+        return P::apply_sign(P::mag(q) == m1 ? r2 : r1, q);
+    }
+};
+template <>
+struct RowOut<F32> {
+    float m2;
+    uint32_t sum;
+    __device__ __forceinline__ RowOut(float a1, float a2, uint32_t negall, const LaunchParams &)
+        : m2(a2), sum(other_sum(a1, a2, negall << 31)) {}
+    __device__ __forceinline__ float operator()(float q, const LaunchParams &p, float scale) const
+    {
+        return __fmul_rn(scale, other_min(q, m2, sum));
+    }
+    __device__ __forceinline__ float operator()(float q, const LaunchParams &p) const { return (*this)(q, p, p.alpha); }
+};
 
 // ---------------------------------------------------------------------------------------------
 // Check-node step (Alg. 1, CN processing) of one check, fused with the stop test of the previous
@@ -304,26 +348,15 @@ __device__ __forceinline__ int check_step(int c, int M, int deg, uint32_t pw, bo
         uint32_t sx;                               // bit 31: parity of the signs
         row_minima<P, DC, UNIFORM>(q, deg, m1, m2, sx);
         const uint32_t negall = ((pw >> 1) ^ (sx >> 31)) & 1u;   // (-1)^{s_m} * prod of all signs
-        if constexpr (LEARNED) {
-            if (w) {
-#pragma unroll
-                for (int j = 0; j < DC; ++j) {
-                    if (UNIFORM || j < deg) {
-                        const mag_t mu = P::mag(q[j]) == m1 ? m2 : m1;   // min over the others
-                        const mag_t r = __fmul_rn(__ldg(w + j * M + c), mu);
-                        slots[j * M + c] = typename P::msg_t(P::signed_like(r, q[j], negall));
-                    }
-                }
-                return (pw & 1u) == 0;
-            }
-        }
-        // alpha * min over the others (r2 where |q_j| is the minimum), with the check's sign factor
-        const mag_t r1 = P::presign(P::scale(m1, p), negall);
-        const mag_t r2 = P::presign(P::scale(m2, p), negall);
+        const RowOut<P> out(m1, m2, negall, p);
 #pragma unroll
         for (int j = 0; j < DC; ++j) {
-            if (UNIFORM || j < deg)
-                slots[j * M + c] = typename P::msg_t(P::apply_sign(P::mag(q[j]) == m1 ? r2 : r1, q[j]));
+            if (UNIFORM || j < deg) {
+                if constexpr (LEARNED)
+                    slots[j * M + c] = out(q[j], p, w ? __ldg(w + j * M + c) : p.alpha);
+                else
+                    slots[j * M + c] = typename P::msg_t(out(q[j], p));
+            }
         }
     }
     return (pw & 1u) == 0;

@@ -46,12 +46,11 @@ __device__ __forceinline__ void layered_check(int c, int M, int deg, uint32_t s_
     }
     mag_t m1, m2;
     row_minima<P, DC, UNIFORM>(q, deg, m1, m2, sx);
-    const uint32_t negall = (s_bit ^ (sx >> 31)) & 1u;
-    const mag_t r1 = P::presign(P::scale(m1, p), negall), r2 = P::presign(P::scale(m2, p), negall);
+    const RowOut<P> out(m1, m2, (s_bit ^ (sx >> 31)) & 1u, p);
 #pragma unroll
     for (int j = 0; j < DC; ++j) {
         if (UNIFORM || j < deg) {
-            const acc_t r = P::apply_sign(P::mag(q[j]) == m1 ? r2 : r1, q[j]);
+            const acc_t r = out(q[j], p);
             Q[v[j]] = P::add(qu[j], r);
             slots[j * M + c] = P::to_msg(r);
         }
@@ -266,13 +265,11 @@ __device__ __forceinline__ int layered_reg_shot(const LayeredOwned<DC, MAXL> &o,
                         }
                         mag_t m1, m2;
                         row_minima<P, D, UNIFORM>(q, o.mdeg[l], m1, m2, sx);
-                        const uint32_t negall = (((sbits >> l) & 1u) ^ (sx >> 31)) & 1u;
-                        const mag_t r1 = P::presign(P::scale(m1, p), negall);
-                        const mag_t r2 = P::presign(P::scale(m2, p), negall);
+                        const RowOut<P> out(m1, m2, (((sbits >> l) & 1u) ^ (sx >> 31)) & 1u, p);
 #pragma unroll
                         for (int j = 0; j < D; ++j) {
                             if (UNIFORM || j < o.mdeg[l]) {
-                                r[l][j] = P::apply_sign(P::mag(q[j]) == m1 ? r2 : r1, q[j]);
+                                r[l][j] = out(q[j], p);
                                 Q[v[j]] = P::add(qu[j], r[l][j]);
                             }
                         }

@@ -231,6 +231,17 @@ __device__ __forceinline__ float2 add2_rn(float2 a, float2 b)
     return o;
 }
 
+__device__ __forceinline__ float2 mul2_rn(float2 a, float2 b)
+{
+    unsigned long long x, y, r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(a.x), "f"(a.y));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(y) : "f"(b.x), "f"(b.y));
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
+    float2 o;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(o.x), "=f"(o.y) : "l"(r));
+    return o;
+}
+
 template <int DC, bool UNIFORM>
 __device__ __forceinline__ void check_step_f32x2(int c, int M, int deg, uint32_t pw, float2 *__restrict__ slots,
                                                  float alpha)
@@ -251,15 +262,11 @@ __device__ __forceinline__ void check_step_f32x2(int c, int M, int deg, uint32_t
     row_minima<P, DC, UNIFORM>(q1, deg, b1, b2, sx1);
     // the check's factor (-1)^{s_m} prod of the signs as a sign bit per lane (pw bit 15 / 31: s_m)
     const uint32_t na = (sx0 ^ (pw << 16)) & 0x80000000u, nb = (sx1 ^ pw) & 0x80000000u;
-    const float ra1 = __uint_as_float(__float_as_uint(__fmul_rn(alpha, a1)) ^ na);
-    const float ra2 = __uint_as_float(__float_as_uint(__fmul_rn(alpha, a2)) ^ na);
-    const float rb1 = __uint_as_float(__float_as_uint(__fmul_rn(alpha, b1)) ^ nb);
-    const float rb2 = __uint_as_float(__float_as_uint(__fmul_rn(alpha, b2)) ^ nb);
+    const uint32_t sa = other_sum(a1, a2, na), sb = other_sum(b1, b2, nb);
 #pragma unroll
     for (int j = 0; j < DC; ++j) {
         if (UNIFORM || j < deg)
-            slots[j * M + c] = make_float2(P::apply_sign(fabsf(q0[j]) == a1 ? ra2 : ra1, q0[j]),
-                                           P::apply_sign(fabsf(q1[j]) == b1 ? rb2 : rb1, q1[j]));
+            slots[j * M + c] = mul2_rn(make_float2(alpha, alpha), make_float2(other_min(q0[j], a2, sa), other_min(q1[j], b2, sb)));
     }
 }
 
