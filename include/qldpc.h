@@ -391,8 +391,8 @@ enum { QLDPC_LOSS_ERROR = 0, QLDPC_LOSS_SYNDROME = 1 };
 QLDPC_API int qldpc_graph_set_weights(qldpc_graph *g, const float *weights, int32_t T);
 
 /* Device workspace (bytes) that qldpc_nms_forward / qldpc_nms_backward need for `batch` shots and
- * T iterations: the slot-layout weights, 16 bytes of recorded state per check, iteration and shot,
- * and the slot-layout gradient.  INVALID_ARG: null pointers, batch < 1, T < 1. */
+ * T iterations: the weights (each row padded to whole groups of two or four edges), 16 bytes of
+ * recorded state per check, iteration and shot, and the gradient in the same layout.  INVALID_ARG: null pointers, batch < 1, T < 1. */
 QLDPC_API int qldpc_nms_workspace_bytes(const qldpc_graph *g, int32_t batch, int32_t T, size_t *bytes);
 
 /*

@@ -285,26 +285,26 @@ cudaError_t launch_msa_learned(const LaunchParams &p, const KernelChoice &kc, di
                                size_t smem, cudaStream_t stream);
 
 // ---------------------------------------------------------------------------------------------
-// Training of the learned decoder (nms_train.cu); the error sampler and the logical test (evaluate.cu).
+// Training of the learned decoder (nms_train.cuh); the error sampler and the logical test (evaluate.cu).
 // ---------------------------------------------------------------------------------------------
-// Recorded check-node state of one iteration: 4 words per check, word f of check i at f*m + i:
-//   0: min1 (FP32 bits)  1: min2 (FP32 bits)  2: sign bits, bit j = [q_j < 0]
-//   3: idx1 | idx2 << 8 | negall << 16   (negall = s_i XOR parity of all sign bits)
-constexpr int kStateWords = 4;
-constexpr int kTrainThreads = 128;   // threads per training block (one shot per block)
+// Recorded check-node state of one iteration: 16 bytes per check,
+//   x: min1 (FP32 bits)  y: min2 (FP32 bits)  z: sign bits, bit j = [q_j < 0]
+//   w: idx1 | idx2 << 8 | negall << 16   (negall = s_i XOR parity of all sign bits)
+constexpr int kTrainThreads = 256;   // most threads of a training block
 
 struct TrainParams {
     DeviceGraph g;
     const uint8_t *syn;         // [batch * m]
     const uint8_t *target;      // [batch * n] true error bits, caller's variable order
     const float *prior;         // [n]
-    const float *w;             // [T][dc_max * m] slot-layout weights
-    uint32_t *state;            // [batch][T][kStateWords * m]
+    const float *w;             // [T][m * wstride] weights in edge groups (train_edge_at)
+    int32_t wstride;            // dc_max rounded up to whole groups
+    uint4 *state;               // [batch][T][m]
     float *loss;                // [batch]
     float *post;                // [batch * n] a-posteriori LLR of iteration T, or nullptr
     const float *grad_loss;     // [batch]
     const float *loss_w;        // [T] per-iteration loss weights lambda_t, or nullptr for 1/T each
-    float *partial;             // [T][dc_max * m] slot-layout weight gradient, zeroed before the backward
+    float *partial;             // [T][m * wstride] weight gradient in edge groups, zeroed before the backward
     int32_t T, batch;
     int32_t loss_kind;          // kLossError or kLossSyndrome
 };
@@ -312,21 +312,29 @@ struct TrainParams {
 constexpr int kLossError = 0;      // BCE of sigma(-Q) against the sampled error, mean over variables
 constexpr int kLossSyndrome = 1;   // BCE of the soft syndrome against s, mean over checks
 
+// Edges of a group in the training kernels' weights and gradients, for a compiled row degree: 2 where groups of 4
+// would leave two or three places of a row's last group empty.
+__host__ __device__ constexpr int train_group(int dc, bool uniform) { return uniform && (dc % 4 == 1 || dc % 4 == 2) ? 2 : 4; }
+// Place of edge j of check i among m checks.
+__host__ __device__ constexpr size_t train_edge_at(int group, int i, int j, int m)
+{
+    return (size_t(j / group) * size_t(m) + size_t(i)) * size_t(group) + size_t(j % group);
+}
+
 struct TrainChoice {
     int dc;          // exact uniform row degree 6..8, else bucket 8/16/32
     bool uniform;
     int dvb;         // column-degree bucket 4/8/16
 };
 
-const void *nms_forward_kernel_ptr(const TrainChoice &tc, int loss_kind);
-const void *nms_backward_kernel_ptr(const TrainChoice &tc, int loss_kind);
-cudaError_t launch_nms_forward(const TrainParams &p, const TrainChoice &tc, int grid, int threads, size_t smem,
-                               cudaStream_t stream);
-cudaError_t launch_nms_backward(const TrainParams &p, const TrainChoice &tc, int grid, int threads, size_t smem,
-                                cudaStream_t stream);
-cudaError_t launch_permute_weights(const float *w_csr, const uint32_t *eslot, int32_t T, int32_t nnz, int32_t S,
-                                   float *w_slot, cudaStream_t stream);
-cudaError_t launch_gather_grad(const float *grad_slot, const uint32_t *eslot, int32_t T, int32_t S, int32_t nnz,
+// Kernels of one (x1) or two (x2) shots per block; nullptr: no such variant.
+const void *train_kernel_x1(const TrainChoice &tc, int loss_kind, bool backward);
+const void *train_kernel_x2(const TrainChoice &tc, int loss_kind, bool backward);
+cudaError_t launch_training(const void *kernel, const TrainParams &p, int grid, int threads, size_t smem,
+                            cudaStream_t stream);
+cudaError_t launch_permute_weights(const float *w_csr, const DeviceGraph &g, int32_t T, int32_t wstride, int group,
+                                   float *w_groups, cudaStream_t stream);
+cudaError_t launch_gather_grad(const float *grad_groups, const DeviceGraph &g, int32_t T, int32_t wstride, int group,
                                float *grad, cudaStream_t stream);
 cudaError_t launch_adam(float *param, const float *grad, float *m1, float *m2, int64_t count, int32_t step,
                         float lr, float beta1, float beta2, float eps, cudaStream_t stream);
@@ -348,25 +356,23 @@ cudaError_t launch_logical(const LogicalPlan &pl, const uint8_t *logicals, int32
                            const uint8_t *dec, const uint8_t *ok, int32_t batch, uint8_t *fail, int sm_count,
                            cudaStream_t stream);
 
-// Shared memory of one training shot (forward: q slots, gamma, targets, syndrome; backward adds
-// the recomputed r slots and the recorded state of two iterations).  The syndrome loss adds the
-// per-edge codes to the forward and Q per lane to the backward, whose codes overwrite r in place.
+// Shared memory of a training block of `shots` shots (n = variable lanes).  Forward: the messages, the codes per
+// edge (syndrome loss), the priors, targets and syndrome bits.  Backward: the gradient slots, the r slots
+// (the syndrome loss's codes overwrite them in place), the code per lane (syndrome loss), and the rest.
 struct TrainLayout {
-    size_t slot_off, r_off, c_off, t_off, g_off, y_off, s_off, total;
+    size_t slot_off, r_off, q_off, g_off, y_off, s_off, total;
 };
 
-__host__ __device__ inline TrainLayout train_layout(int m, int n, int dc_max, bool backward, bool syndrome = false)
+__host__ __device__ inline TrainLayout train_layout(int m, int n, int dc_max, int shots, bool backward, bool syndrome)
 {
     TrainLayout t;
-    const size_t S = size_t(dc_max) * m + kScratch;
-    t.slot_off = 0;                                                          // q / gradient slots [S] f32
-    t.r_off = align16(S * 4);                                                // r slots [S] f32 (backward)
-    t.c_off = backward ? align16(t.r_off + S * 4) : t.r_off;                 // state [2][4m] u32 (backward)
-    t.t_off = backward ? align16(t.c_off + 2 * size_t(kStateWords) * m * 4) : t.c_off;   // syndrome loss:
-    const size_t g0 = syndrome ? align16(t.t_off + (backward ? size_t(n) : S) * 4) : t.t_off; // codes [S] / Q [n]
-    t.g_off = g0;                                                                        // gamma [n] f32
-    t.y_off = align16(t.g_off + size_t(n) * 4);                              // targets [n] u8
-    t.s_off = align16(t.y_off + size_t(n));                                  // syndrome bits [m] u8
+    const size_t W = 4 * size_t(shots), S = align16((size_t(dc_max) * m + kScratch) * W);
+    t.slot_off = 0;
+    t.r_off = S;
+    t.q_off = t.r_off + (backward || syndrome ? S : 0);
+    t.g_off = t.q_off + (backward && syndrome ? align16(size_t(n) * W) : 0);
+    t.y_off = align16(t.g_off + size_t(n) * 4);                 // targets [n] u8, bit l: shot l
+    t.s_off = align16(t.y_off + (syndrome ? 0 : size_t(n)));    // syndrome bits [m] u8, bit l: shot l
     t.total = align16(t.s_off + size_t(m));
     return t;
 }

@@ -1,0 +1,734 @@
+// Training of the neural normalized min-sum decoder on sm_103a: Algorithm 1 (Sec. 2 of
+// arXiv 2508.07879) with the scale alpha replaced by a learned weight w[t][e] per iteration and
+// edge, unrolled over T iterations, trained on the BCE of the soft outputs sigma(-Q).
+//
+//   nms_forward_kernel   T iterations of the learned check step and the exact variable step of the decoder
+//                        kernels (so FP32 messages are bit-identical to the learned decoder's), the per-shot
+//                        loss sum_t lambda_t / N sum_n BCE(sigma(-Q^t_n), y_n) (lambda_t = 1/T unless
+//                        given), and, per iteration and check, the
+//                        compressed check state: min1, min2, the positions attaining them (lowest on
+//                        ties), the sign bits of the inputs and the syndrome-flipped total sign.
+//   nms_backward_kernel  the reverse sweep.  It stores no message: every r^(t) is recomputed from
+//                        the recorded state (r_{m,n} = sign * (w * (n == idx1 ? min2 : min1))),
+//                        Q^(t) from those r, and the gradient flows
+//                          dL/dr_{m,n}   = dL/dQ_n + sum_{i != m} dL/dq_{i,n}      (variable step)
+//                          dL/dw_{m,n}   = dL/dr_{m,n} * sign * min_{j != n}|q_j|
+//                          dL/dq_{m,idx1} = sum_{n != idx1} dL/dr_{m,n} w sign * sign(q_idx1)
+//                          dL/dq_{m,idx2} = dL/dr_{m,idx1} w sign * sign(q_idx2)     (all other q: 0)
+//                        Weight gradients are added into one L2-resident buffer with global
+//                        reductions, so the order of the sum over shots follows the schedule: the
+//                        last bits of a gradient can differ between calls.
+//
+// L = 1 or 2 shots per block.  Two shots share every weight, edge list and prior, their messages sit in one
+// 8-byte slot per edge (as in the two-shots-per-block decoder), their sums and products are packed FP32
+// operations.  Weights and their gradient lie in groups of four edges (two where a row's length asks for it), so a
+// check moves four of them per instruction and a warp whole sectors.  Each shot's gradient is added by itself: adding the pair first halves the
+// reductions but changes the order of the sum over shots, whose rounding is the largest error of a gradient.
+// What bounds both kernels is instruction issue and the latency of short chains between barriers, not
+// memory: the recorded state (16 bytes per check, iteration and shot, written once and read from L2 after
+// a prefetch) and the gradient's reductions are the only traffic.
+// LP-1054, 4096 shots, T = 20, syndrome loss: forward 1097 -> 528 us, backward 2664 -> 872 us
+// (error loss 784 -> 619 and 1687 -> 679).
+#pragma once
+
+#include <cstdint>
+#include <type_traits>
+
+#include <cuda_runtime.h>
+
+#include "msa_kernel.cuh"
+#include "msa_launch.h"
+
+namespace qldpc {
+namespace kern {
+
+// ---------------------------------------------------------------------------------------------
+// The same number of L shots: a float or a pair, with lane-wise operations rounded to nearest
+// ---------------------------------------------------------------------------------------------
+template <int L>
+struct Lanes {
+    using word = float;
+    static __device__ __forceinline__ word all(float x) { return x; }
+    static __device__ __forceinline__ word add(word a, word b) { return __fadd_rn(a, b); }
+    static __device__ __forceinline__ word sub(word a, word b) { return __fsub_rn(a, b); }
+    static __device__ __forceinline__ word mul(word a, word b) { return __fmul_rn(a, b); }
+    static __device__ __forceinline__ word fma(word a, word b, word c) { return __fmaf_rn(a, b, c); }
+    static __device__ __forceinline__ float get(word a, int) { return a; }
+    static __device__ __forceinline__ void set(word &a, int, float x) { a = x; }
+};
+#define QLDPC_PACKED2(name, op)                                                                 \
+    static __device__ __forceinline__ word name(word a, word b)                                 \
+    {                                                                                           \
+        unsigned long long x, y, r;                                                             \
+        asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(a.x), "f"(a.y));                            \
+        asm("mov.b64 %0, {%1, %2};" : "=l"(y) : "f"(b.x), "f"(b.y));                            \
+        asm(op " %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));                                      \
+        word o;                                                                                 \
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(o.x), "=f"(o.y) : "l"(r));                           \
+        return o;                                                                               \
+    }
+template <>
+struct Lanes<2> {
+    using word = float2;
+    static __device__ __forceinline__ word all(float x) { return make_float2(x, x); }
+    QLDPC_PACKED2(add, "add.rn.f32x2")
+    QLDPC_PACKED2(mul, "mul.rn.f32x2")
+    static __device__ __forceinline__ word sub(word a, word b) { return add(a, make_float2(-b.x, -b.y)); }
+    static __device__ __forceinline__ word fma(word a, word b, word c)
+    {
+        unsigned long long x, y, z, r;
+        asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(a.x), "f"(a.y));
+        asm("mov.b64 %0, {%1, %2};" : "=l"(y) : "f"(b.x), "f"(b.y));
+        asm("mov.b64 %0, {%1, %2};" : "=l"(z) : "f"(c.x), "f"(c.y));
+        asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(x), "l"(y), "l"(z));
+        word o;
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(o.x), "=f"(o.y) : "l"(r));
+        return o;
+    }
+    static __device__ __forceinline__ float get(word a, int l) { return l ? a.y : a.x; }
+    static __device__ __forceinline__ void set(word &a, int l, float x) { (l ? a.y : a.x) = x; }
+};
+#undef QLDPC_PACKED2
+
+__device__ __forceinline__ float with_sign(float mag, uint32_t bit31) { return __uint_as_float(__float_as_uint(mag) ^ bit31); }
+__device__ __forceinline__ uint32_t sign_of(float x) { return __float_as_uint(x) & 0x80000000u; }
+
+__device__ __forceinline__ float softplus(float x) { return fmaxf(x, 0.0f) + log1pf(expf(-fabsf(x))); }
+__device__ __forceinline__ float sigmoid(float x) { return 1.0f / (1.0f + expf(-x)); }
+
+// Sum over the block (deterministic order); every thread gets the total.
+__device__ __forceinline__ float block_sum(float v, float *red)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
+    __syncthreads();
+    if (lane == 0) red[warp] = v;
+    __syncthreads();
+    float t = 0.0f;
+    for (int i = 0; i < nw; ++i) t += red[i];
+    return t;
+}
+
+// f(D, u) for this thread's variable lanes u = tid, tid + T, ... with their degree D a compile-time constant
+// (lanes come in classes of one degree, as in the two-shots-per-block decoder).
+template <int DV, class F>
+__device__ __forceinline__ void for_lanes(const DeviceGraph &G, int tid, int T, F f)
+{
+    int u = tid;
+    for (int cl = 0; cl < G.ncls && u < G.nv; ++cl) {
+        const int u1 = G.cls_end[cl];
+        auto run = [&](auto deg) {
+#pragma unroll 1
+            for (; u < u1; u += T) f(deg, u);
+        };
+        switch (G.cls_deg[cl]) {
+#define QLDPC_CASE(DD)                                                                          \
+    case DD:                                                                                    \
+        if constexpr (DD <= DV) run(std::integral_constant<int, DD>{});                         \
+        break;
+            QLDPC_DEG_CASES(QLDPC_CASE)
+#undef QLDPC_CASE
+        default:   // a degree above the variant's bucket (the host never launches one)
+            while (u < u1) u += T;
+            break;
+        }
+    }
+}
+
+// Weights and their gradient: the edges of a row in groups of G, a group's values of all checks one after
+// another, so that a warp's 32 checks move whole sectors with one G-wide load or reduction (edge j of check
+// c at edge_at<G>(c, j, M); rows are padded with zeros to whole groups).
+template <int DC, bool UNIFORM>
+__host__ __device__ constexpr int edge_group()
+{
+    return train_group(DC, UNIFORM);
+}
+
+// The weights of check c: DC values, 0 past the row's end.
+template <int DC, bool UNIFORM>
+__device__ __forceinline__ void load_row(const float *__restrict__ rows, int M, int c, int deg, float (&w)[DC])
+{
+    constexpr int G = edge_group<DC, UNIFORM>();
+#pragma unroll
+    for (int j = 0; j < DC; j += G) {
+        float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        if (UNIFORM || j < deg) {
+            const float *at = rows + train_edge_at(G, c, j, M);
+            if constexpr (G == 2) {
+                const float2 x = __ldg(reinterpret_cast<const float2 *>(at));
+                v[0] = x.x;
+                v[1] = x.y;
+            } else {
+                const float4 x = __ldg(reinterpret_cast<const float4 *>(at));
+                v[0] = x.x;
+                v[1] = x.y;
+                v[2] = x.z;
+                v[3] = x.w;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < G; ++i)
+            if (j + i < DC) w[j + i] = v[i];
+    }
+}
+
+// ---------------------------------------------------------------------------------------------
+// Syndrome loss.  With t_v = tanh(Q_v / 2), P_c = (1 + (-1)^s prod_{v in c} t_v) / 2 is the
+// probability that row c's parity under independent bits sigma(-Q) equals s.  Each variable stores on
+// its edge slots its code: u_v = 1 - |t_v| = 2 x / (1 + x), x = e^-|Q_v|, with the sign of Q_v (also on
+// u = 0, where |Q| is so large that |t| = 1).  A check then needs 1 - prod |t| = 1 - prod (1 - u) without
+// the cancellation of the difference: D <- D + u (1 - D) over the row, every term positive.  A violated,
+// confident check gets P = D / 2 exactly as small as it is, a met one P = 1 - D / 2.  One exponential
+// per variable and one logarithm per check; the sum of logarithms this replaces (two log1p a variable,
+// an exp or expm1 a check and an exp per edge of the backward) was most of both kernels.
+// ---------------------------------------------------------------------------------------------
+constexpr float kSynLossFloor = 1e-7f;
+
+__device__ __forceinline__ float soft_code(float Q)
+{
+    const float x = expf(-fabsf(Q));
+    return with_sign(__fdividef(2.0f * x, 1.0f + x), Q < 0.0f ? 0x80000000u : 0u);
+}
+// d tanh(Q/2) / dQ = (1 - t^2) / 2 = u (1 - u / 2)
+__device__ __forceinline__ float code_slope(float code)
+{
+    const float u = fabsf(code);
+    return u * (1.0f - 0.5f * u);
+}
+
+// P_c of L shots from the codes in check c's slots; s_bits: bit l = s_c of shot l.  WANT_T: the signed t_j.
+template <int L, int DC, bool UNIFORM, bool WANT_T>
+__device__ __forceinline__ void parity_match(int c, int M, int deg, uint32_t s_bits,
+                                             const typename Lanes<L>::word *__restrict__ ts, float (&P)[L],
+                                             typename Lanes<L>::word (&t)[DC])
+{
+    using V = Lanes<L>;
+    using word = typename V::word;
+    word D = V::all(0.0f);
+    uint32_t neg[L];
+#pragma unroll
+    for (int l = 0; l < L; ++l) neg[l] = s_bits << (31 - l);
+#pragma unroll
+    for (int j = 0; j < DC; ++j) {
+        if (UNIFORM || j < deg) {
+            const word code = ts[j * M + c];
+            word u;
+#pragma unroll
+            for (int l = 0; l < L; ++l) {
+                neg[l] ^= __float_as_uint(V::get(code, l));
+                V::set(u, l, fabsf(V::get(code, l)));
+            }
+            D = V::fma(u, V::sub(V::all(1.0f), D), D);
+            if constexpr (WANT_T) {
+                const word m = V::sub(V::all(1.0f), u);
+#pragma unroll
+                for (int l = 0; l < L; ++l) V::set(t[j], l, with_sign(V::get(m, l), sign_of(V::get(code, l))));
+            }
+        } else if constexpr (WANT_T) {
+            t[j] = V::all(1.0f);
+        }
+    }
+#pragma unroll
+    for (int l = 0; l < L; ++l) P[l] = (neg[l] >> 31) ? 0.5f * V::get(D, l) : 1.0f - 0.5f * V::get(D, l);
+}
+
+template <int L, int DC, bool UNIFORM>
+__device__ __forceinline__ void syndrome_term(int c, int M, int deg, uint32_t s_bits,
+                                              const typename Lanes<L>::word *__restrict__ ts, float (&term)[L])
+{
+    float P[L];
+    typename Lanes<L>::word none[DC];
+    parity_match<L, DC, UNIFORM, false>(c, M, deg, s_bits, ts, P, none);
+#pragma unroll
+    for (int l = 0; l < L; ++l) term[l] = -logf(fmaxf(P[l], kSynLossFloor));
+}
+
+// d(syndrome term)/d t_j = -(1 / P) (-1)^s / 2 prod_{i != j} t_i (0 at the floor), written over the
+// codes of check c.
+template <int L, int DC, bool UNIFORM>
+__device__ __forceinline__ void syndrome_term_grad(int c, int M, int deg, uint32_t s_bits,
+                                                   typename Lanes<L>::word *__restrict__ ts)
+{
+    using V = Lanes<L>;
+    using word = typename V::word;
+    float P[L];
+    word t[DC], pre[DC];
+    parity_match<L, DC, UNIFORM, true>(c, M, deg, s_bits, ts, P, t);
+    word coef;
+#pragma unroll
+    for (int l = 0; l < L; ++l)
+        V::set(coef, l, P[l] > kSynLossFloor ? ((s_bits >> l) & 1u ? 0.5f : -0.5f) / P[l] : 0.0f);
+    word run = coef;
+#pragma unroll
+    for (int j = 0; j < DC; ++j) {
+        pre[j] = run;                        // coef t_0 ... t_{j-1}
+        run = V::mul(run, t[j]);
+    }
+    word suf = V::all(1.0f);                 // t_{j+1} ... t_{deg-1}
+#pragma unroll
+    for (int j = DC - 1; j >= 0; --j) {
+        if (UNIFORM || j < deg) {
+            ts[j * M + c] = V::mul(pre[j], suf);
+            suf = V::mul(suf, t[j]);
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------------------------
+// Forward
+// ---------------------------------------------------------------------------------------------
+// Learned check step for check c: r = sign * (w * min over the others), written in place of q, and the
+// recorded state of shot l at st[l] (not where st[l] is null).
+template <int L, int DC, bool UNIFORM>
+__device__ __forceinline__ void train_check(int c, int M, int deg, uint32_t s_bits,
+                                            typename Lanes<L>::word *__restrict__ slots, const float *__restrict__ w,
+                                            uint4 *const (&st)[L])
+{
+    using V = Lanes<L>;
+    float q[L][DC], wv[DC], m2[L];
+    uint32_t sum[L];
+    load_row<DC, UNIFORM>(w, M, c, deg, wv);
+#pragma unroll
+    for (int j = 0; j < DC; ++j) {
+        if (UNIFORM || j < deg) {
+            const typename V::word v = slots[j * M + c];
+#pragma unroll
+            for (int l = 0; l < L; ++l) q[l][j] = V::get(v, l);
+        }
+    }
+#pragma unroll
+    for (int l = 0; l < L; ++l) {
+        float m1;
+        uint32_t sx;
+        row_minima<F32, DC, UNIFORM>(q[l], deg, m1, m2[l], sx);
+        const uint32_t negall = ((s_bits >> l) ^ (sx >> 31)) & 1u;
+        sum[l] = other_sum(m1, m2[l], negall << 31);
+        uint32_t signs = 0, at1 = 0, at2 = 0;
+#pragma unroll
+        for (int j = DC - 1; j >= 0; --j) {
+            if (UNIFORM || j < deg) {
+                signs = __funnelshift_l(__float_as_uint(q[l][j]), signs, 1);
+                if (fabsf(q[l][j]) == m1) at1 |= 1u << j;
+                if (fabsf(q[l][j]) == m2[l]) at2 |= 1u << j;
+            }
+        }
+        // the lowest position of the minimum, and the lowest other position of the second smallest (0 where
+        // a NaN hides them, so that an index always names an edge)
+        const int i1 = at1 ? __ffs(int(at1)) - 1 : 0;
+        at2 &= ~(1u << i1);
+        const int i2 = at2 ? __ffs(int(at2)) - 1 : 0;
+        if (st[l])
+            st[l][c] = make_uint4(__float_as_uint(m1), __float_as_uint(m2[l]), signs,
+                                  uint32_t(i1) | (uint32_t(i2) << 8) | (negall << 16));
+    }
+#pragma unroll
+    for (int j = 0; j < DC; ++j) {
+        if (UNIFORM || j < deg) {
+            typename V::word o;
+#pragma unroll
+            for (int l = 0; l < L; ++l) V::set(o, l, other_min(q[l][j], m2[l], sum[l]));
+            slots[j * M + c] = V::mul(V::all(wv[j]), o);
+        }
+    }
+}
+
+// Per-lane inputs: the prior of the variable in lane u, and its targets (bit l: shot l; kIdleLane where the
+// lane holds no variable: its prior is 0, its edges are scratch slots and it adds nothing to the loss).
+constexpr uint8_t kIdleLane = 0x80;
+__device__ __forceinline__ float lane_prior(const DeviceGraph &g, const float *prior, int u)
+{
+    const uint32_t v = __ldg(g.vperm + u);
+    return v < uint32_t(g.n) ? prior[v] : 0.0f;
+}
+template <int L>
+__device__ __forceinline__ uint8_t lane_targets(const DeviceGraph &g, const uint8_t *target, const int (&shot)[L], int u)
+{
+    const uint32_t v = __ldg(g.vperm + u);
+    if (v >= uint32_t(g.n)) return kIdleLane;
+    uint8_t y = 0;
+#pragma unroll
+    for (int l = 0; l < L; ++l) y |= uint8_t((target[size_t(shot[l]) * g.n + v] & 1u) << l);
+    return y;
+}
+
+// The block's shots; one past the batch's end takes the first one's inputs and leaves no output.
+template <int L>
+__device__ __forceinline__ void block_shots(int batch, int (&shot)[L], bool (&real)[L])
+{
+#pragma unroll
+    for (int l = 0; l < L; ++l) {
+        const int64_t b = int64_t(blockIdx.x) * L + l;
+        real[l] = b < batch;
+        shot[l] = real[l] ? int(b) : int(blockIdx.x) * L;
+    }
+}
+
+template <int L>
+__device__ __forceinline__ uint8_t check_bits(const uint8_t *syn, const int (&shot)[L], int M, int c)
+{
+    uint8_t s = 0;
+#pragma unroll
+    for (int l = 0; l < L; ++l) s |= uint8_t((syn[size_t(shot[l]) * M + c] & 1u) << l);
+    return s;
+}
+
+// SYN: the syndrome loss (compiled separately, so the error-loss kernels carry none of its code).
+template <int L, int DC, bool UNIFORM, int DV, bool SYN>
+__global__ void __launch_bounds__(kTrainThreads, DC <= 8 ? 3 : 1) nms_forward_kernel(const __grid_constant__ TrainParams p)
+{
+    using V = Lanes<L>;
+    using word = typename V::word;
+    const DeviceGraph &G = p.g;
+    const int M = G.m, N = G.n, NV = G.nv, T = blockDim.x, tid = threadIdx.x;
+    extern __shared__ __align__(16) unsigned char smem[];
+    const TrainLayout lay = train_layout(M, NV, G.dc_max, L, false, SYN);
+    word *slots = reinterpret_cast<word *>(smem + lay.slot_off);
+    word *ts = reinterpret_cast<word *>(smem + lay.r_off);        // syndrome loss: each edge's variable's code
+    float *gam = reinterpret_cast<float *>(smem + lay.g_off);
+    uint8_t *y = smem + lay.y_off;
+    uint8_t *sb = smem + lay.s_off;
+    __shared__ float red[32];
+    int shot[L];
+    bool real[L];
+    block_shots<L>(p.batch, shot, real);
+
+    for (int c = tid; c < M; c += T) sb[c] = check_bits<L>(p.syn, shot, M, c);
+    for_lanes<DV>(G, tid, T, [&](auto deg, int u) {
+        constexpr int D = decltype(deg)::value;
+        const float g = F32::quantize(lane_prior(G, p.prior, u));
+        gam[u] = g;
+        if constexpr (!SYN) y[u] = lane_targets<L>(G, p.target, shot, u);
+#pragma unroll
+        for (int i = 0; i < D; ++i) slots[__ldg(G.vslot16 + i * NV + u)] = V::all(g);
+    });
+    __syncthreads();
+    float acc[L];
+#pragma unroll
+    for (int l = 0; l < L; ++l) acc[l] = 0.0f;
+    // uniform lambda: sum the terms and scale once by 1/(T K); else weight each iteration's terms
+    // (K = N variables for the error loss, M checks for the syndrome loss)
+    const float K = float(SYN ? M : N);
+    const float inv = p.loss_w ? 1.0f / K : 1.0f / (float(p.T) * K);
+    for (int k = 0; k < p.T; ++k) {
+        const float *wk = p.w + size_t(k) * M * p.wstride;
+        uint4 *st[L];
+#pragma unroll
+        for (int l = 0; l < L; ++l) st[l] = real[l] ? p.state + (size_t(shot[l]) * p.T + k) * M : nullptr;
+        // syndrome loss of iteration k-1 (its code slots are complete) beside the check step of k
+        const float lw_prev = (SYN && k > 0) ? (p.loss_w ? __ldg(p.loss_w + k - 1) : 1.0f) : 0.0f;
+        for (int c = tid; c < M; c += T) {
+            const int deg = UNIFORM ? DC : int(__ldg(G.rdeg + c));
+            if (SYN && k > 0) {
+                float term[L];
+                syndrome_term<L, DC, UNIFORM>(c, M, deg, sb[c], ts, term);
+#pragma unroll
+                for (int l = 0; l < L; ++l) acc[l] += lw_prev * term[l];
+            }
+            train_check<L, DC, UNIFORM>(c, M, deg, sb[c], slots, wk, st);
+        }
+        __syncthreads();
+        const bool lastk = k + 1 == p.T;
+        const float lw = p.loss_w ? __ldg(p.loss_w + k) : 1.0f;
+        for_lanes<DV>(G, tid, T, [&](auto deg, int u) {
+            constexpr int D = decltype(deg)::value;
+            uint32_t e[D > 0 ? D : 1];
+            word r[D > 0 ? D : 1], pre[D + 1];
+#pragma unroll
+            for (int i = 0; i < D; ++i) e[i] = __ldg(G.vslot16 + i * NV + u);
+#pragma unroll
+            for (int i = 0; i < D; ++i) r[i] = slots[e[i]];
+            pre[0] = V::all(gam[u]);
+#pragma unroll
+            for (int i = 0; i < D; ++i) pre[i + 1] = V::add(pre[i], r[i]);
+            const word Q = pre[D];
+#pragma unroll
+            for (int i = 0; i < D; ++i) {
+                word q = pre[i];
+#pragma unroll
+                for (int h = i + 1; h < D; ++h) q = V::add(q, r[h]);
+                slots[e[i]] = q;
+            }
+            if constexpr (SYN) {
+                word code;
+#pragma unroll
+                for (int l = 0; l < L; ++l) V::set(code, l, soft_code(V::get(Q, l)));
+#pragma unroll
+                for (int i = 0; i < D; ++i) ts[e[i]] = code;
+            } else if (y[u] != kIdleLane) {
+#pragma unroll
+                for (int l = 0; l < L; ++l) {
+                    const float q = V::get(Q, l);
+                    acc[l] += lw * ((y[u] >> l) & 1u ? softplus(q) : softplus(-q));
+                }
+            }
+            if (lastk && p.post) {
+                const uint32_t v = __ldg(G.vperm + u);
+#pragma unroll
+                for (int l = 0; l < L; ++l)
+                    if (v < uint32_t(N) && real[l]) p.post[size_t(shot[l]) * N + v] = V::get(Q, l);
+            }
+        });
+        __syncthreads();
+    }
+    if (SYN) {   // the last iteration's syndrome loss
+        const float lw = p.loss_w ? __ldg(p.loss_w + p.T - 1) : 1.0f;
+        for (int c = tid; c < M; c += T) {
+            float term[L];
+            syndrome_term<L, DC, UNIFORM>(c, M, UNIFORM ? DC : int(__ldg(G.rdeg + c)), sb[c], ts, term);
+#pragma unroll
+            for (int l = 0; l < L; ++l) acc[l] += lw * term[l];
+        }
+    }
+#pragma unroll
+    for (int l = 0; l < L; ++l) {
+        const float total = block_sum(acc[l], red);
+        if (tid == 0 && real[l]) p.loss[shot[l]] = total * inv;
+    }
+}
+
+// ---------------------------------------------------------------------------------------------
+// Backward
+// ---------------------------------------------------------------------------------------------
+// Bring one iteration's recorded state (16 bytes per check) of a shot into L2.
+__device__ __forceinline__ void prefetch_state(const uint4 *st, int M, int tid, int T)
+{
+    for (int i = 8 * tid; i < M; i += 8 * T) asm volatile("prefetch.global.L2 [%0];" ::"l"(st + i));
+}
+
+// r of check c recomputed from its recorded state and its edges' weights (bit-identical to the
+// forward's r).
+template <int L, int DC, bool UNIFORM>
+__device__ __forceinline__ void recompute_r(int c, int M, int deg, const uint4 (&st)[L], const float (&w)[DC],
+                                            typename Lanes<L>::word *__restrict__ rs)
+{
+    using V = Lanes<L>;
+    uint32_t flip[L];
+#pragma unroll
+    for (int l = 0; l < L; ++l) flip[l] = st[l].z ^ (0u - ((st[l].w >> 16) & 1u));   // bit j: the sign of r_j
+#pragma unroll
+    for (int j = 0; j < DC; ++j) {
+        if (UNIFORM || j < deg) {
+            typename V::word mu;
+#pragma unroll
+            for (int l = 0; l < L; ++l)
+                V::set(mu, l, with_sign(__uint_as_float(j == int(st[l].w & 0xffu) ? st[l].y : st[l].x),
+                                        (flip[l] << (31 - j)) & 0x80000000u));
+            rs[j * M + c] = V::mul(V::all(w[j]), mu);
+        }
+    }
+}
+
+template <int L, int DC, bool UNIFORM, int DV, bool SYN>
+__global__ void __launch_bounds__(kTrainThreads, DC <= 8 ? 3 : 1) nms_backward_kernel(const __grid_constant__ TrainParams p)
+{
+    using V = Lanes<L>;
+    using word = typename V::word;
+    const DeviceGraph &G = p.g;
+    const int M = G.m, N = G.n, NV = G.nv, T = blockDim.x, tid = threadIdx.x;
+    const size_t S = size_t(M) * p.wstride;
+    extern __shared__ __align__(16) unsigned char smem[];
+    const TrainLayout lay = train_layout(M, NV, G.dc_max, L, true, SYN);
+    word *gs = reinterpret_cast<word *>(smem + lay.slot_off);     // dL/dq (next iteration), then dL/dr
+    word *rs = reinterpret_cast<word *>(smem + lay.r_off);        // recomputed r of the current iteration
+    // Syndrome loss: once Q^(k) is formed, each variable overwrites its own r slots with its code
+    // (no other thread reads them), and each check then replaces the codes with d(term)/d t.
+    word *ts = rs;
+    word *ucode = reinterpret_cast<word *>(smem + lay.q_off);     // syndrome loss: the code per lane
+    float *gam = reinterpret_cast<float *>(smem + lay.g_off);
+    uint8_t *y = smem + lay.y_off;
+    uint8_t *sb = smem + lay.s_off;
+    int shot[L];
+    bool real[L];
+    block_shots<L>(p.batch, shot, real);
+    const uint4 *st[L];
+    word gscale;
+#pragma unroll
+    for (int l = 0; l < L; ++l) {
+        st[l] = p.state + size_t(shot[l]) * p.T * M;
+        V::set(gscale, l, real[l] ? p.grad_loss[shot[l]] * (1.0f / float(SYN ? M : N)) : 0.0f);
+        if (p.T > 1) prefetch_state(st[l] + size_t(p.T - 2) * M, M, tid, T);
+    }
+
+    // iteration T: recompute r; dL/dq of iteration T+1 is zero
+    for (int c = tid; c < M; c += T) {
+        const int deg = UNIFORM ? DC : int(__ldg(G.rdeg + c));
+        if (SYN) sb[c] = check_bits<L>(p.syn, shot, M, c);
+        float w[DC];
+        uint4 s[L];
+#pragma unroll
+        for (int l = 0; l < L; ++l) s[l] = __ldg(st[l] + size_t(p.T - 1) * M + c);
+        load_row<DC, UNIFORM>(p.w + size_t(p.T - 1) * S, M, c, deg, w);
+        recompute_r<L, DC, UNIFORM>(c, M, deg, s, w, rs);
+#pragma unroll
+        for (int j = 0; j < DC; ++j)
+            if (UNIFORM || j < deg) gs[j * M + c] = V::all(0.0f);
+    }
+    for (int u = tid; u < NV; u += T) {
+        gam[u] = F32::quantize(lane_prior(G, p.prior, u));
+        if constexpr (!SYN) y[u] = lane_targets<L>(G, p.target, shot, u);
+    }
+    __syncthreads();
+    for (int k = p.T - 1; k >= 0; --k) {
+        if (k > 1) {
+#pragma unroll
+            for (int l = 0; l < L; ++l) prefetch_state(st[l] + size_t(k - 2) * M, M, tid, T);
+        }
+        const word gk = V::mul(gscale, V::all(p.loss_w ? __ldg(p.loss_w + k) : 1.0f / float(p.T)));
+        if constexpr (SYN) {
+            // the code of Q^(k) on every edge slot, then each check's d(loss term)/d t in its place
+            for_lanes<DV>(G, tid, T, [&](auto deg, int u) {
+                constexpr int D = decltype(deg)::value;
+                uint32_t e[D > 0 ? D : 1];
+#pragma unroll
+                for (int i = 0; i < D; ++i) e[i] = __ldg(G.vslot16 + i * NV + u);
+                word Q = V::all(gam[u]), code;
+#pragma unroll
+                for (int i = 0; i < D; ++i) Q = V::add(Q, rs[e[i]]);
+#pragma unroll
+                for (int l = 0; l < L; ++l) V::set(code, l, soft_code(V::get(Q, l)));
+                ucode[u] = code;
+#pragma unroll
+                for (int i = 0; i < D; ++i) ts[e[i]] = code;
+            });
+            __syncthreads();
+            for (int c = tid; c < M; c += T)
+                syndrome_term_grad<L, DC, UNIFORM>(c, M, UNIFORM ? DC : int(__ldg(G.rdeg + c)), sb[c], ts);
+            __syncthreads();
+        }
+        // variable side: dL/dQ^(k) (error loss: Q^(k) from the recomputed r), and dL/dr for every edge
+        for_lanes<DV>(G, tid, T, [&](auto deg, int u) {
+            constexpr int D = decltype(deg)::value;
+            uint32_t e[D > 0 ? D : 1];
+            word g[D > 0 ? D : 1], sum = V::all(0.0f), gQ;
+#pragma unroll
+            for (int i = 0; i < D; ++i) e[i] = __ldg(G.vslot16 + i * NV + u);
+#pragma unroll
+            for (int i = 0; i < D; ++i) {
+                g[i] = gs[e[i]];
+                sum = V::add(sum, g[i]);
+            }
+            if constexpr (SYN) {
+                word H = V::all(0.0f), slope;
+#pragma unroll
+                for (int i = 0; i < D; ++i) H = V::add(H, ts[e[i]]);
+                const word code = ucode[u];
+#pragma unroll
+                for (int l = 0; l < L; ++l) V::set(slope, l, code_slope(V::get(code, l)));
+                gQ = V::mul(V::mul(gk, slope), H);
+            } else {
+                word Q = V::all(gam[u]);
+#pragma unroll
+                for (int i = 0; i < D; ++i) Q = V::add(Q, rs[e[i]]);
+#pragma unroll
+                for (int l = 0; l < L; ++l)
+                    V::set(gQ, l, V::get(gk, l) * (float((y[u] >> l) & 1u) - sigmoid(-V::get(Q, l))));
+            }
+#pragma unroll
+            for (int i = 0; i < D; ++i) gs[e[i]] = V::add(gQ, V::sub(sum, g[i]));
+        });
+        __syncthreads();
+        // check side: weight gradient, dL/dq of iteration k, and r of iteration k-1
+        for (int c = tid; c < M; c += T) {
+            const int deg = UNIFORM ? DC : int(__ldg(G.rdeg + c));
+            constexpr int GW = edge_group<DC, UNIFORM>(), PAD = (DC + GW - 1) / GW * GW;
+            float w[DC], dw[L][PAD];
+            uint4 s[L], sp[L];
+#pragma unroll
+            for (int l = 0; l < L; ++l) s[l] = __ldg(st[l] + size_t(k) * M + c);
+            load_row<DC, UNIFORM>(p.w + size_t(k) * S, M, c, deg, w);
+            if (k > 0) {
+#pragma unroll
+                for (int l = 0; l < L; ++l) sp[l] = __ldg(st[l] + size_t(k - 1) * M + c);
+            }
+            uint32_t flip[L];
+            float rest[L], own[L];     // sum of gr w sign over the edges but idx1, and idx1's
+#pragma unroll
+            for (int l = 0; l < L; ++l) {
+                flip[l] = s[l].z ^ (0u - ((s[l].w >> 16) & 1u));
+                rest[l] = own[l] = 0.0f;
+            }
+#pragma unroll
+            for (int j = 0; j < PAD; ++j) {
+#pragma unroll
+                for (int l = 0; l < L; ++l) dw[l][j] = 0.0f;
+                if (j < DC && (UNIFORM || j < deg)) {
+                    const word gr = gs[j * M + c];
+                    word sg;           // gr * sign
+#pragma unroll
+                    for (int l = 0; l < L; ++l) V::set(sg, l, with_sign(V::get(gr, l), (flip[l] << (31 - j)) & 0x80000000u));
+                    const word t = V::mul(sg, V::all(w[j]));
+#pragma unroll
+                    for (int l = 0; l < L; ++l) {
+                        const bool min1 = j == int(s[l].w & 0xffu);
+                        dw[l][j] = __fmul_rn(V::get(sg, l), __uint_as_float(min1 ? s[l].y : s[l].x));
+                        if (min1)
+                            own[l] = V::get(t, l);
+                        else
+                            rest[l] += V::get(t, l);
+                    }
+                    gs[j * M + c] = V::all(0.0f);
+                }
+            }
+            float *out = p.partial + size_t(k) * S;
+#pragma unroll
+            for (int l = 0; l < L; ++l)
+#pragma unroll
+                for (int j = 0; j < PAD; j += GW)     // (results unused: reductions; 0 past the row's end)
+                    if (real[l] && (UNIFORM || j < deg)) {
+                        float *at = out + train_edge_at(GW, c, j, M);
+                        if constexpr (GW == 2)
+                            atomicAdd(reinterpret_cast<float2 *>(at), make_float2(dw[l][j], dw[l][j + 1]));
+                        else
+                            atomicAdd(reinterpret_cast<float4 *>(at),
+                                      make_float4(dw[l][j], dw[l][j + 1], dw[l][j + 2], dw[l][j + 3]));
+                    }
+            // dL/dq is 0 but at the positions of the two minima
+            float *g1 = reinterpret_cast<float *>(gs);
+#pragma unroll
+            for (int l = 0; l < L; ++l) {
+                const int i1 = int(s[l].w & 0xffu), i2 = int((s[l].w >> 8) & 0xffu);
+                g1[(i1 * M + c) * L + l] = (s[l].z >> i1) & 1u ? -rest[l] : rest[l];
+                g1[(i2 * M + c) * L + l] = (s[l].z >> i2) & 1u ? -own[l] : own[l];
+            }
+            if (k > 0) {
+                load_row<DC, UNIFORM>(p.w + size_t(k - 1) * S, M, c, deg, w);
+                recompute_r<L, DC, UNIFORM>(c, M, deg, sp, w, rs);
+            }
+        }
+        __syncthreads();
+    }
+}
+
+}  // namespace kern
+
+// Compiled training variants: uniform row degree 6..8 with column-degree bucket 4 or 8, or a row-degree
+// bucket 8 with column-degree bucket 8 or 16 (both for one and two shots per block); longer rows take one
+// shot per block.
+#define QLDPC_TRAIN_SHORT(X)                                                                    \
+    X(6, true, 4) X(6, true, 8) X(7, true, 4) X(7, true, 8) X(8, true, 4) X(8, true, 8)        \
+    X(8, false, 8) X(8, false, 16)
+#define QLDPC_TRAIN_LONG(X) X(16, false, 8) X(16, false, 16) X(32, false, 8) X(32, false, 16)
+
+template <int L, bool BACKWARD>
+const void *train_kernel(const TrainChoice &tc, int loss_kind)
+{
+    const bool syn = loss_kind == kLossSyndrome;
+#define QLDPC_K(DCV, UNI, DVV)                                                                  \
+    if (tc.dc == DCV && tc.uniform == UNI && tc.dvb == DVV) {                                   \
+        if constexpr (BACKWARD)                                                                 \
+            return syn ? reinterpret_cast<const void *>(&kern::nms_backward_kernel<L, DCV, UNI, DVV, true>) \
+                       : reinterpret_cast<const void *>(&kern::nms_backward_kernel<L, DCV, UNI, DVV, false>); \
+        else                                                                                    \
+            return syn ? reinterpret_cast<const void *>(&kern::nms_forward_kernel<L, DCV, UNI, DVV, true>) \
+                       : reinterpret_cast<const void *>(&kern::nms_forward_kernel<L, DCV, UNI, DVV, false>); \
+    }
+    QLDPC_TRAIN_SHORT(QLDPC_K)
+    if constexpr (L == 1) {
+        QLDPC_TRAIN_LONG(QLDPC_K)
+    }
+#undef QLDPC_K
+    return nullptr;
+}
+
+}  // namespace qldpc

@@ -1,6 +1,6 @@
 // Host side of the learned-decoder entry points of include/qldpc.h: weight upload for learned
 // decoding, workspace sizing, argument validation and launches of the training kernels
-// (nms_train.cu), the Adam step, the device error sampler and the logical-failure test.  No
+// (nms_train.cuh), the Adam step, the device error sampler and the logical-failure test.  No
 // arithmetic of the method runs here.
 #include "qldpc.h"
 
@@ -24,7 +24,7 @@ constexpr size_t kAlign = 256;
 
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
-// Compiled training variant for a graph (see nms_train.cu), or dc = -1 if none.
+// Compiled training variant for a graph (see nms_train.cuh), or dc = -1 if none.
 TrainChoice train_choice(const qldpc_graph *g)
 {
     const int dvb = dv_bucket(g->dv_max);
@@ -36,9 +36,10 @@ TrainChoice train_choice(const qldpc_graph *g)
 
 struct TrainPlan {
     TrainChoice tc{};
-    const void *fwd[2] = {nullptr, nullptr}, *bwd[2] = {nullptr, nullptr};   // [loss kind]
-    size_t smem_f[2] = {0, 0}, smem_b[2] = {0, 0};   // [loss kind]
-    int grid_f[2] = {0, 0}, grid_b[2] = {0, 0};
+    int shots = 1, threads = 0, grid = 0;            // per block; blocks
+    const void *kernel[2][2] = {};                   // [loss kind][backward]
+    size_t smem[2][2] = {};
+    int32_t wstride = 0, group = 4;
     size_t w_off = 0, state_off = 0, part_off = 0, total = 0;
 };
 
@@ -62,36 +63,46 @@ int plan_training(const qldpc_graph *g, int32_t batch, int32_t T, TrainPlan &tp)
     return QLDPC_OK;
 }
 
+// Two shots per block share weights, edge lists and reductions, where they fit and every SM still gets
+// several blocks; below that the batch is spread one shot per block (LP-1054, T = 20, syndrome loss, one
+// against two shots per block, forward + backward us: 456 shots 254 | 285, 608 shots 349 | 295, 4096 shots
+// 1693 | 1399; 72 checks on 144 variables, 608 shots 120 | 125, 1216 shots 151 | 146).
+constexpr int kPairShotsPerSm = 3;
+
+int plan_kernels(const qldpc_graph *g, TrainPlan &tp)
+{
+    for (int kind = 0; kind < 2; ++kind)
+        for (int back = 0; back < 2; ++back) {
+            tp.kernel[kind][back] = tp.shots == 2 ? train_kernel_x2(tp.tc, kind, back) : train_kernel_x1(tp.tc, kind, back);
+            if (!tp.kernel[kind][back]) return QLDPC_ERR_UNSUPPORTED;
+            tp.smem[kind][back] = train_layout(g->m, g->nv, g->dc_max, tp.shots, back, kind == kLossSyndrome).total;
+            if (int rc = ensure_kernel_attrs(tp.kernel[kind][back], tp.smem[kind][back], g->smem_optin)) return rc;
+        }
+    return QLDPC_OK;
+}
+
 int plan_training_uncached(const qldpc_graph *g, int32_t batch, int32_t T, TrainPlan &tp)
 {
     tp.tc = train_choice(g);
     if (tp.tc.dc < 0) return QLDPC_ERR_UNSUPPORTED;
-    for (int kind = 0; kind < 2; ++kind) {
-        const bool syn = kind == kLossSyndrome;
-        tp.fwd[kind] = nms_forward_kernel_ptr(tp.tc, kind);
-        tp.bwd[kind] = nms_backward_kernel_ptr(tp.tc, kind);
-        if (!tp.fwd[kind] || !tp.bwd[kind]) return QLDPC_ERR_UNSUPPORTED;
-        tp.smem_f[kind] = train_layout(g->m, g->nv, g->dc_max, false, syn).total;
-        tp.smem_b[kind] = train_layout(g->m, g->nv, g->dc_max, true, syn).total;
-        if (int rc = ensure_kernel_attrs(tp.fwd[kind], tp.smem_f[kind], g->smem_optin)) return rc;
-        if (int rc = ensure_kernel_attrs(tp.bwd[kind], tp.smem_b[kind], g->smem_optin)) return rc;
+    if (!g->dg.vslot16) return QLDPC_ERR_UNSUPPORTED;   // (more edge slots than any training block holds)
+    tp.shots = int64_t(batch) > int64_t(kPairShotsPerSm) * g->sm_count ? 2 : 1;
+    int rc = plan_kernels(g, tp);
+    if (rc == QLDPC_ERR_UNSUPPORTED && tp.shots == 2) {
+        tp.shots = 1;
+        rc = plan_kernels(g, tp);
     }
-    for (int kind = 0; kind < 2; ++kind) {
-        int per_f = 0, per_b = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_f, tp.fwd[kind], kTrainThreads, tp.smem_f[kind]) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_b, tp.bwd[kind], kTrainThreads, tp.smem_b[kind]) != cudaSuccess) {
-            cudaGetLastError();
-            return QLDPC_ERR_CUDA;
-        }
-        if (per_f < 1 || per_b < 1) return QLDPC_ERR_UNSUPPORTED;
-        tp.grid_f[kind] = int(std::min<int64_t>(batch, int64_t(per_f) * g->sm_count));
-        tp.grid_b[kind] = int(std::min<int64_t>(batch, int64_t(per_b) * g->sm_count));
-    }
-    const size_t S = size_t(g->dc_max) * size_t(g->m);
+    if (rc) return rc;
+    // threads: one pass over the checks of a small code
+    tp.threads = std::min(kTrainThreads, std::max(64, (g->m + 31) / 32 * 32));
+    tp.grid = int((int64_t(batch) + tp.shots - 1) / tp.shots);
+    tp.group = train_group(tp.tc.dc, tp.tc.uniform);
+    tp.wstride = (g->dc_max + tp.group - 1) / tp.group * tp.group;
+    const size_t rows = size_t(T) * size_t(g->m) * size_t(tp.wstride) * sizeof(float);
     tp.w_off = 0;
-    tp.state_off = align_up(size_t(T) * S * sizeof(float));
-    tp.part_off = tp.state_off + align_up(size_t(batch) * size_t(T) * kStateWords * size_t(g->m) * sizeof(uint32_t));
-    tp.total = tp.part_off + align_up(size_t(T) * S * sizeof(float));
+    tp.state_off = align_up(rows);
+    tp.part_off = tp.state_off + align_up(size_t(batch) * size_t(T) * size_t(g->m) * sizeof(uint4));
+    tp.total = tp.part_off + align_up(rows);
     return QLDPC_OK;
 }
 
@@ -111,7 +122,8 @@ TrainParams train_params(const qldpc_graph *g, const TrainPlan &tp, const uint8_
     p.target = target;
     p.prior = prior;
     p.w = reinterpret_cast<const float *>(b + tp.w_off);
-    p.state = reinterpret_cast<uint32_t *>(b + tp.state_off);
+    p.wstride = tp.wstride;
+    p.state = reinterpret_cast<uint4 *>(b + tp.state_off);
     p.partial = reinterpret_cast<float *>(b + tp.part_off);
     p.T = T;
     p.batch = batch;
@@ -192,10 +204,8 @@ int qldpc_nms_forward(const qldpc_graph *g, const uint8_t *syndromes, const uint
     p.post = out_post;
     p.loss_w = loss_weights;
     p.loss_kind = loss;
-    const size_t S = size_t(g->dc_max) * size_t(g->m);
-    cudaError_t e = launch_permute_weights(weights, g->dg.eslot, T, g->nnz, int32_t(S),
-                                           const_cast<float *>(p.w), st);
-    if (e == cudaSuccess) e = launch_nms_forward(p, tp.tc, tp.grid_f[loss], kTrainThreads, tp.smem_f[loss], st);
+    cudaError_t e = launch_permute_weights(weights, g->dg, T, tp.wstride, tp.group, const_cast<float *>(p.w), st);
+    if (e == cudaSuccess) e = launch_training(tp.kernel[loss][0], p, tp.grid, tp.threads, tp.smem[loss][0], st);
     return cuda_status(e);
 }
 
@@ -217,10 +227,9 @@ int qldpc_nms_backward(const qldpc_graph *g, const uint8_t *syndromes, const uin
     p.grad_loss = grad_loss;
     p.loss_w = loss_weights;
     p.loss_kind = loss;
-    const size_t S = size_t(g->dc_max) * size_t(g->m);
-    cudaError_t e = cudaMemsetAsync(p.partial, 0, size_t(T) * S * sizeof(float), st);
-    if (e == cudaSuccess) e = launch_nms_backward(p, tp.tc, tp.grid_b[loss], kTrainThreads, tp.smem_b[loss], st);
-    if (e == cudaSuccess) e = launch_gather_grad(p.partial, g->dg.eslot, T, int32_t(S), g->nnz, out_grad, st);
+    cudaError_t e = cudaMemsetAsync(p.partial, 0, tp.total - tp.part_off, st);
+    if (e == cudaSuccess) e = launch_training(tp.kernel[loss][1], p, tp.grid, tp.threads, tp.smem[loss][1], st);
+    if (e == cudaSuccess) e = launch_gather_grad(p.partial, g->dg, T, tp.wstride, tp.group, out_grad, st);
     return cuda_status(e);
 }
 
