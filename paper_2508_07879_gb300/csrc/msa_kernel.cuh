@@ -5,10 +5,10 @@
 //
 //   msa_batch_kernel    throughput: one block per shot, persistent over the batch, one thread per
 //                       check in the check step and one thread per variable in the variable step;
-//                       edge lists are read through the read-only path (L1-resident).
-//   msa_latency_kernel  single-shot latency: the same steps, but every thread keeps its edge
+//                       16-bit edge lists are read through the read-only path (L1-resident).
+//   msa_latency_kernel  single shots and moderate batches: the same steps, but every thread keeps its edge
 //                       lists, degrees, priors and a-posteriori LLRs in registers for the whole
-//                       decode, so an iteration touches only shared memory.
+//                       launch, so an iteration touches only shared memory.
 //
 // Layout (a GB300 design, not the paper's per-iteration launches over global memory):
 //   * every edge message of a shot lives in shared memory, in place: the check step overwrites
@@ -137,6 +137,18 @@ struct IFix {
 };
 using I16 = IFix<int16_t, 8, 32767>;
 using I8 = IFix<int8_t, 2, 127>;
+
+// The same arithmetic with 4-byte slots.  The variable lanes are packed so that a warp's slots fall in distinct
+// 4-byte banks; 2- and 1-byte slots share banks (1.5 wavefronts an access on LP-1054) and need conversions.  The
+// single-shot kernel, whose shared memory is never short, keeps its messages so.
+template <class P>
+struct WideSlots {
+    using type = P;
+};
+template <class MSG, int FRAC, int LIM>
+struct WideSlots<IFix<MSG, FRAC, LIM>> {
+    using type = IFix<int32_t, FRAC, LIM>;
+};
 
 template <class P>
 __device__ __forceinline__ typename P::acc_t load_msg(const typename P::msg_t *s, uint32_t i)
@@ -404,74 +416,82 @@ __device__ __forceinline__ typename P::acc_t var_step_exact(const uint32_t *sl, 
 
 #define QLDPC_DEG_CASES(X) X(0) X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11) X(12) X(13) X(14) X(15) X(16)
 
-// Batch variant: the edge list comes from global memory (L1-resident).
-template <class P, int D, bool TRACK = true>
-__device__ __forceinline__ typename P::acc_t var_step_global(int v, int N, const CheckOf &ck, const uint32_t *__restrict__ vslot,
-                                                             typename P::acc_t gamma, bool prev,
-                                                             typename P::msg_t *slots, uint32_t *parity)
+// f(D, u) for this thread's variable lanes u = tid, tid + T, ... with their degree D a compile-time constant
+// (lanes come in classes of one degree, walked in order; reading each lane's degree and branching on it costs
+// a tenth of a decode).
+template <int DV, class F>
+__device__ __forceinline__ void for_lanes(const DeviceGraph &G, int tid, int T, F f)
 {
-    uint32_t e[D > 0 ? D : 1];
-#pragma unroll
-    for (int k = 0; k < D; ++k) e[k] = __ldg(vslot + size_t(k) * N + v);
-    return var_step_exact<P, D, TRACK>(e, ck, gamma, prev, slots, parity);
+    int u = tid;
+    for (int cl = 0; cl < G.ncls && u < G.nv; ++cl) {
+        const int u1 = G.cls_end[cl];
+        auto run = [&](auto deg) {
+#pragma unroll 1
+            for (; u < u1; u += T) f(deg, u);
+        };
+        switch (G.cls_deg[cl]) {
+#define QLDPC_CASE(DD)                                                                          \
+    case DD:                                                                                    \
+        if constexpr (DD <= DV) run(std::integral_constant<int, DD>{});                         \
+        break;
+            QLDPC_DEG_CASES(QLDPC_CASE)
+#undef QLDPC_CASE
+        default:   // a degree above the variant's bucket (the host never launches one)
+            while (u < u1) u += T;
+            break;
+        }
+    }
 }
 
-// Variable step of the batch kernel for one variable: dispatch on its degree (internal variables
-// are sorted by degree, so the lanes of a warp almost always take the same case).
-template <class P, int DV, bool TRACK = true>
-__device__ __forceinline__ typename P::acc_t var_step_batch(int deg, int u, int N, const CheckOf &ck, const uint32_t *vslot,
-                                                            typename P::acc_t gamma, bool prev,
-                                                            typename P::msg_t *slots, uint32_t *parity)
+// The edge list of lane u from the 16-bit lists, or from the 32-bit ones on a graph with more slots than they
+// index (no such graph fits a block in FP32).
+template <int D, bool WIDE>
+__device__ __forceinline__ void lane_edges(const DeviceGraph &g, int u, uint32_t (&e)[D > 0 ? D : 1])
 {
-    switch (deg) {
-#define QLDPC_CASE(D)                                                                           \
-    case D:                                                                                     \
-        if constexpr (D <= DV) return var_step_global<P, D, TRACK>(u, N, ck, vslot, gamma, prev, slots, parity); \
-        break;
-        QLDPC_DEG_CASES(QLDPC_CASE)
-#undef QLDPC_CASE
-    default: break;
-    }
-    return gamma;
+#pragma unroll
+    for (int k = 0; k < D; ++k) e[k] = WIDE ? __ldg(g.vslot + size_t(k) * g.nv + u) : uint32_t(__ldg(g.vslot16 + k * g.nv + u));
 }
 
 // ---------------------------------------------------------------------------------------------
 // Throughput kernel
 // ---------------------------------------------------------------------------------------------
 // Initialization (Alg. 1) of one shot: q^(0) = gamma on every edge; the parity words start at s_m
-// and take the decisions of the prior.  Ends with a barrier.  N = variable lanes.
-template <class P>
-__device__ __forceinline__ void batch_init_shot(const Problem &pr, const uint8_t *s, int M, int N, int tid, int T,
+// and take the decisions of the prior.  Ends with a barrier.
+template <class P, int DV, bool WIDE>
+__device__ __forceinline__ void batch_init_shot(const DeviceGraph &g, const uint8_t *s, int tid, int T,
                                                 const typename P::acc_t *gam, typename P::acc_t *Qs,
                                                 uint32_t *parity, typename P::msg_t *slots)
 {
-    for (int c = tid; c < M; c += T) parity[c] = (s[c] & 1u) * 3u;
+    for (int c = tid; c < g.m; c += T) parity[c] = (s[c] & 1u) * 3u;
     __syncthreads();
-    const CheckOf ck(pr.g);
-    for (int u = tid; u < N; u += T) {
-        const typename P::acc_t g = gam[u];
-        const int deg = __ldg(pr.g.vdeg + u);
-        const bool d = P::neg(g);
-        for (int k = 0; k < deg; ++k) {
-            const uint32_t e = __ldg(pr.g.vslot + size_t(k) * N + u);
-            slots[e] = P::to_msg(g);
-            if (d) flip_check(parity, ck(e));
+    const CheckOf ck(g);
+    for_lanes<DV>(g, tid, T, [&](auto deg, int u) {
+        constexpr int D = decltype(deg)::value;
+        uint32_t e[D > 0 ? D : 1];
+        lane_edges<D, WIDE>(g, u, e);
+        const typename P::acc_t x = gam[u];
+        const bool d = P::neg(x);
+#pragma unroll
+        for (int k = 0; k < D; ++k) {
+            slots[e[k]] = P::to_msg(x);
+            if (d) flip_check(parity, ck(e[k]));
         }
-        Qs[u] = g;
-    }
+        Qs[u] = x;
+    });
     __syncthreads();
 }
 
 // LEARNED: iterations 1..learned_iters use the learned weights; a shot whose syndrome is still not
 // met then restarts from its prior with plain min-sum (alpha) for up to max_iter iterations, and
 // reports learned_iters + the plain iterations.  Learned launches always stop early.
-template <class P, int DC, bool UNIFORM, int DV, bool LEARNED = false>
-__global__ void __launch_bounds__(1024, 1) msa_batch_kernel(const LaunchParams p)
+template <class P, int DC, bool UNIFORM, int DV, bool LEARNED, bool WIDE>
+__device__ __forceinline__ void batch_decode(const LaunchParams &p)
 {
     using acc_t = typename P::acc_t;
     using msg_t = typename P::msg_t;
 
     const Problem pr = blockIdx.y == 0 ? p.prob[0] : p.prob[1];
+    const DeviceGraph &G = p.prob[blockIdx.y].g;   // read in place (the class tables are indexed at run time)
     const int M = pr.g.m, N = pr.g.n, NV = pr.g.nv;   // checks, variables, variable lanes
     const int T = blockDim.x, tid = threadIdx.x;
 
@@ -521,7 +541,7 @@ __global__ void __launch_bounds__(1024, 1) msa_batch_kernel(const LaunchParams p
             continue;
         }
         const uint8_t *s = pr.syn + size_t(b) * M;
-        batch_init_shot<P>(pr, s, M, NV, tid, T, gam, Qs, parity, slots);
+        batch_init_shot<P, DV, WIDE>(G, s, tid, T, gam, Qs, parity, slots);
 
         int k = 0, all = 0;
         bool learned = LEARNED;
@@ -541,23 +561,24 @@ __global__ void __launch_bounds__(1024, 1) msa_batch_kernel(const LaunchParams p
                 if (!LEARNED || !learned) break;
                 learned = false;                  // fallback: plain min-sum from the prior
                 end = k + p.max_iter;
-                batch_init_shot<P>(pr, s, M, NV, tid, T, gam, Qs, parity, slots);
+                batch_init_shot<P, DV, WIDE>(G, s, tid, T, gam, Qs, parity, slots);
                 continue;
             }
-            for (int u = tid; u < NV; u += T)
-                Qs[u] = var_step_batch<P, DV>(__ldg(pr.g.vdeg + u), u, NV, CheckOf(pr.g), pr.g.vslot, gam[u],
-                                              P::neg(Qs[u]), slots, parity);
+            const CheckOf ck(pr.g);
+            for_lanes<DV>(G, tid, T, [&](auto deg, int u) {
+                constexpr int D = decltype(deg)::value;
+                uint32_t e[D > 0 ? D : 1];
+                lane_edges<D, WIDE>(G, u, e);
+                Qs[u] = var_step_exact<P, D>(e, ck, gam[u], P::neg(Qs[u]), slots, parity);
+            });
             __syncthreads();
             ++k;
         }
 
-        for (int u = tid; u < NV; u += T) {
-            const acc_t q = Qs[u];
-            const uint32_t v = __ldg(pr.g.vperm + u);
-            if (v < uint32_t(N)) {
-                err[v] = P::neg(q) ? 1 : 0;
-                if (pr.post) pr.post[size_t(b) * N + v] = P::post(q);
-            }
+        for (int v = tid; v < N; v += T) {   // in variable order: a warp's stores are adjacent
+            const acc_t q = Qs[__ldg(pr.g.vlane + v)];
+            err[v] = P::neg(q) ? 1 : 0;
+            if (pr.post) pr.post[size_t(b) * N + v] = P::post(q);
         }
         if (tid == 0) {
             pr.iters[b] = k;
@@ -565,6 +586,17 @@ __global__ void __launch_bounds__(1024, 1) msa_batch_kernel(const LaunchParams p
         }
         __syncthreads();   // the next shot reuses shared memory
     }
+}
+
+template <class P, int DC, bool UNIFORM, int DV, bool LEARNED = false>
+__global__ void __launch_bounds__(1024, 1) msa_batch_kernel(const __grid_constant__ LaunchParams p)
+{
+    if constexpr (sizeof(typename P::msg_t) < 4)
+        if (!p.prob[blockIdx.y].g.vslot16) {
+            batch_decode<P, DC, UNIFORM, DV, LEARNED, true>(p);
+            return;
+        }
+    batch_decode<P, DC, UNIFORM, DV, LEARNED, false>(p);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -590,7 +622,10 @@ __device__ __forceinline__ typename P::acc_t var_step_regs(int deg, const uint32
     return gamma;
 }
 
-template <class P, int DC, bool UNIFORM, int DV, bool LEARNED = false>
+// PT: checks and variable lanes per thread, 1 where a block of at most kLatencyMaxThreads covers both, else 2.  With
+// one of each a thread needs 48 to 64 registers instead of 72 to 94, so two to eight blocks share an SM: 65536 shots of
+// the 144 x 288 code FP32 861 -> 690 us (and INT16 with 4-byte slots 1322 -> 794), 6400 of the 192 x 400 code 352 -> 338.
+template <class P, int DC, bool UNIFORM, int DV, int PT, bool LEARNED = false>
 __global__ void __launch_bounds__(kLatencyMaxThreads, 1) msa_latency_kernel(const LaunchParams p)
 {
     using acc_t = typename P::acc_t;
@@ -605,20 +640,20 @@ __global__ void __launch_bounds__(kLatencyMaxThreads, 1) msa_latency_kernel(cons
     msg_t *slots = reinterpret_cast<msg_t *>(smem + L.slot_off);
 
     // Checks c = tid + i*T: degree in registers.
-    int cdeg[kLatCnPerThread];
+    int cdeg[PT];
 #pragma unroll
-    for (int i = 0; i < kLatCnPerThread; ++i) {
+    for (int i = 0; i < PT; ++i) {
         const int c = tid + i * T;
         cdeg[i] = c < M ? (UNIFORM ? DC : int(__ldg(pr.g.rdeg + c))) : -1;
     }
     // Variable lanes u = tid + i*T (heaviest first, so the few second-pass variables are the
     // lightest): edge lists, degree and prior in registers; vid = original index for the outputs.
-    uint32_t ev[kLatVnPerThread][DV];
-    int vdeg[kLatVnPerThread], vid[kLatVnPerThread];
-    acc_t gam[kLatVnPerThread];
+    uint32_t ev[PT][DV];
+    int vdeg[PT], vid[PT];
+    acc_t gam[PT];
     int bad = 0;
 #pragma unroll
-    for (int i = 0; i < kLatVnPerThread; ++i) {
+    for (int i = 0; i < PT; ++i) {
         const int u = tid + i * T;
         const int v = u < NV ? int(__ldg(pr.g.vperm + u)) : N;   // N: idle lane
         vid[i] = v;
@@ -634,11 +669,20 @@ __global__ void __launch_bounds__(kLatencyMaxThreads, 1) msa_latency_kernel(cons
 
     const bool early = LEARNED || (p.flags & kFlagNoEarlyStop) == 0;
     const size_t wstride = size_t(pr.g.dc_max) * M;
-    for (int b = blockIdx.x; b < p.batch; b += gridDim.x) {
+    __shared__ int s_shot[2];   // alternating claim words, as in the batch kernel
+    int claim = 0;
+    for (int b = blockIdx.x;; b += gridDim.x) {
+        if (p.next_shot) {      // more shots than blocks
+            if (tid == 0) s_shot[claim] = atomicAdd(p.next_shot + blockIdx.y, 1);
+            __syncthreads();
+            b = s_shot[claim];
+            claim ^= 1;
+        }
+        if (b >= p.batch) break;
         uint8_t *err = pr.err + size_t(b) * N;
         if (bad) {
 #pragma unroll
-            for (int i = 0; i < kLatVnPerThread; ++i) {
+            for (int i = 0; i < PT; ++i) {
                 const int v = vid[i];
                 if (v < N) {
                     err[v] = 0;
@@ -652,15 +696,15 @@ __global__ void __launch_bounds__(kLatencyMaxThreads, 1) msa_latency_kernel(cons
             continue;
         }
         const uint8_t *s = pr.syn + size_t(b) * M;
-        acc_t Q[kLatVnPerThread];
+        acc_t Q[PT];
         // Initialization (Alg. 1), also the restart of the plain fallback; ends with a barrier.
         auto init_shot = [&]() {
 #pragma unroll
-            for (int i = 0; i < kLatCnPerThread; ++i)
+            for (int i = 0; i < PT; ++i)
                 if (cdeg[i] >= 0) parity[tid + i * T] = (s[tid + i * T] & 1u) * 3u;
             __syncthreads();
 #pragma unroll
-            for (int i = 0; i < kLatVnPerThread; ++i) {
+            for (int i = 0; i < PT; ++i) {
                 Q[i] = gam[i];
                 const bool d = P::neg(gam[i]);
 #pragma unroll
@@ -684,7 +728,7 @@ __global__ void __launch_bounds__(kLatencyMaxThreads, 1) msa_latency_kernel(cons
             if constexpr (LEARNED) wk = (learned && !last) ? pr.weights + size_t(k) * wstride : nullptr;
             int ok = 1;
 #pragma unroll
-            for (int i = 0; i < kLatCnPerThread; ++i)
+            for (int i = 0; i < PT; ++i)
                 if (cdeg[i] >= 0)
                     ok &= check_step<P, DC, UNIFORM, LEARNED>(tid + i * T, M, cdeg[i], parity[tid + i * T], !last,
                                                               slots, p, wk);
@@ -698,7 +742,7 @@ __global__ void __launch_bounds__(kLatencyMaxThreads, 1) msa_latency_kernel(cons
                 continue;
             }
 #pragma unroll
-            for (int i = 0; i < kLatVnPerThread; ++i)
+            for (int i = 0; i < PT; ++i)
                 if (vdeg[i] >= 0)
                     Q[i] = var_step_regs<P, DV>(vdeg[i], ev[i], CheckOf(pr.g), gam[i], P::neg(Q[i]), slots, parity);
             __syncthreads();
@@ -706,7 +750,7 @@ __global__ void __launch_bounds__(kLatencyMaxThreads, 1) msa_latency_kernel(cons
         }
 
 #pragma unroll
-        for (int i = 0; i < kLatVnPerThread; ++i) {
+        for (int i = 0; i < PT; ++i) {
             const int v = vid[i];
             if (v < N) {
                 err[v] = P::neg(Q[i]) ? 1 : 0;
@@ -736,10 +780,12 @@ __global__ void __launch_bounds__(kLatencyMaxThreads, 1) msa_latency_kernel(cons
 template <class P, bool LEARNED = false>
 const void *kernel_table(const KernelChoice &kc)
 {
+    using W = typename kern::WideSlots<P>::type;   // (the single-shot kernel's slots: latency_layout with 4 bytes)
 #define QLDPC_K(DCV, UNI, DVV)                                                                  \
     if (kc.dc == DCV && kc.uniform == UNI && kc.dvb == DVV)                                     \
-        return kc.latency ? reinterpret_cast<const void *>(&kern::msa_latency_kernel<P, DCV, UNI, DVV, LEARNED>) \
-                          : reinterpret_cast<const void *>(&kern::msa_batch_kernel<P, DCV, UNI, DVV, LEARNED>);
+        return !kc.latency      ? reinterpret_cast<const void *>(&kern::msa_batch_kernel<P, DCV, UNI, DVV, LEARNED>) \
+               : kc.one_pass    ? reinterpret_cast<const void *>(&kern::msa_latency_kernel<W, DCV, UNI, DVV, 1, LEARNED>) \
+                                : reinterpret_cast<const void *>(&kern::msa_latency_kernel<W, DCV, UNI, DVV, 2, LEARNED>);
     QLDPC_VARIANTS(QLDPC_K)
 #undef QLDPC_K
     return nullptr;
@@ -749,17 +795,11 @@ template <class P, bool LEARNED = false>
 cudaError_t launch_table(const LaunchParams &p, const KernelChoice &kc, dim3 grid, int threads,
                          size_t smem, cudaStream_t stream)
 {
-#define QLDPC_L(DCV, UNI, DVV)                                                                  \
-    if (kc.dc == DCV && kc.uniform == UNI && kc.dvb == DVV) {                                   \
-        if (kc.latency)                                                                         \
-            kern::msa_latency_kernel<P, DCV, UNI, DVV, LEARNED><<<grid, threads, smem, stream>>>(p); \
-        else                                                                                    \
-            kern::msa_batch_kernel<P, DCV, UNI, DVV, LEARNED><<<grid, threads, smem, stream>>>(p); \
-        return cudaGetLastError();                                                              \
-    }
-    QLDPC_VARIANTS(QLDPC_L)
-#undef QLDPC_L
-    return cudaErrorInvalidValue;
+    const void *k = kernel_table<P, LEARNED>(kc);
+    if (!k) return cudaErrorInvalidValue;
+    void *args[] = {const_cast<LaunchParams *>(&p)};
+    const cudaError_t e = cudaLaunchKernel(k, grid, dim3(unsigned(threads)), args, smem, stream);
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace qldpc

@@ -132,6 +132,7 @@ struct KernelChoice {
     int dvb;         // column-degree bucket 4/8/16
     bool learned = false;   // learned weights first, then plain fallback (FP32 only)
     bool layered = false;   // msa_layered_kernel (row-serial schedule)
+    bool one_pass = false;  // latency kernel with one check and one variable lane per thread (else two)
     bool packed = false;    // msa_packed_kernel: two fixed-point shots per message word (INT16 / INT8)
 };
 
@@ -140,6 +141,7 @@ struct KernelChoice {
 constexpr int kLatencyCnPerThread = 2;
 constexpr int kLatencyVnPerThread = 2;
 constexpr int kLatencyMaxThreads = 640;
+constexpr int kLatencySlotBytes = 4;   // in every precision (WideSlots)
 
 // ---------------------------------------------------------------------------------------------
 // Persistent server (server_kernel.cuh): worker blocks that take requests of any code from one

@@ -110,32 +110,6 @@ __device__ __forceinline__ float block_sum(float v, float *red)
     return t;
 }
 
-// f(D, u) for this thread's variable lanes u = tid, tid + T, ... with their degree D a compile-time constant
-// (lanes come in classes of one degree, as in the two-shots-per-block decoder).
-template <int DV, class F>
-__device__ __forceinline__ void for_lanes(const DeviceGraph &G, int tid, int T, F f)
-{
-    int u = tid;
-    for (int cl = 0; cl < G.ncls && u < G.nv; ++cl) {
-        const int u1 = G.cls_end[cl];
-        auto run = [&](auto deg) {
-#pragma unroll 1
-            for (; u < u1; u += T) f(deg, u);
-        };
-        switch (G.cls_deg[cl]) {
-#define QLDPC_CASE(DD)                                                                          \
-    case DD:                                                                                    \
-        if constexpr (DD <= DV) run(std::integral_constant<int, DD>{});                         \
-        break;
-            QLDPC_DEG_CASES(QLDPC_CASE)
-#undef QLDPC_CASE
-        default:   // a degree above the variant's bucket (the host never launches one)
-            while (u < u1) u += T;
-            break;
-        }
-    }
-}
-
 // Weights and their gradient: the edges of a row in groups of G, a group's values of all checks one after
 // another, so that a warp's 32 checks move whole sectors with one G-wide load or reduction (edge j of check
 // c at edge_at<G>(c, j, M); rows are padded with zeros to whole groups).

@@ -603,7 +603,7 @@ int plan_latency(const qldpc_graph *const *gs, int nprob, int32_t batch, int pre
     for (int i = 0; i < nprob; ++i) {
         one = std::max(one, round32(std::max(gs[i]->m, gs[i]->nv)));
         two = std::max(two, round32(std::max((gs[i]->m + 1) / 2, (gs[i]->nv + 1) / 2)));
-        smem = std::max(smem, latency_layout(gs[i]->m, gs[i]->dc_max, msg_bytes(precision)).total);
+        smem = std::max(smem, latency_layout(gs[i]->m, gs[i]->dc_max, kLatencySlotBytes).total);
     }
     const int threads = (forced && g0->user_threads) ? g0->user_threads
                                                       : (one <= kLatencyMaxThreads ? one : two);
@@ -612,6 +612,8 @@ int plan_latency(const qldpc_graph *const *gs, int nprob, int32_t batch, int pre
         fits = fits && gs[i]->m <= kLatencyCnPerThread * threads && gs[i]->nv <= kLatencyVnPerThread * threads;
     if (!fits) return forced ? QLDPC_ERR_UNSUPPORTED : QLDPC_OK;
     pl.kc = variant(gs, nprob, true, learned);
+    pl.kc.one_pass = true;
+    for (int i = 0; i < nprob; ++i) pl.kc.one_pass = pl.kc.one_pass && gs[i]->m <= threads && gs[i]->nv <= threads;
     pl.threads = threads;
     pl.smem = smem;
     const void *k = msa_kernel(precision, pl.kc);
@@ -742,7 +744,7 @@ int launch(const qldpc_graph *g0, const qldpc_graph *g1, const Problem *probs, i
             if (int rc = plan_batch(gs, nprob, batch, precision, learned, pl)) return rc;
     }
     if (plan_only) return QLDPC_OK;
-    if (!latency && (pl.kc.packed || pl.grid < batch)) {
+    if (pl.kc.packed || pl.grid < batch) {
         // more shots than blocks (or the packed kernel, whose lanes always take shots from a counter):
         // claim them dynamically from a zeroed counter pair of the ring
         p.next_shot = g0->d_counters + 2 * size_t(g0->counter_seq.fetch_add(1) % kShotCounterSlots);
