@@ -528,9 +528,11 @@ struct Plan {
 
 int round32(int x) { return (x + 31) / 32 * 32; }
 
-// Threads per block of the batch kernel: measured within 3 % of the best block size on the
-// 192-, 465- and 144-check codes (several small blocks per SM beat few large ones).
-constexpr int kBatchThreads = 128;
+// Shots of a call that each SM decodes.
+int64_t shots_per_sm(const qldpc_graph *g0, int nprob, int32_t batch)
+{
+    return (int64_t(batch) * nprob + g0->sm_count - 1) / g0->sm_count;
+}
 
 // Compiled variant for the graphs of one call: exact uniform row degree 6..9, else a bucket.
 KernelChoice variant(const qldpc_graph *const *gs, int nprob, bool latency, bool learned)
@@ -587,9 +589,18 @@ int occupancy_grid(const qldpc_graph *g0, const void *k, int threads, size_t sme
     return QLDPC_OK;
 }
 
-// Single-shot (latency) path: chosen automatically when every shot of the call gets its own SM,
-// or forced with QLDPC_KERNEL_LATENCY.  One pass over the checks and the variables when both fit
+// Single-shot (latency) path: one pass over the checks and the variables when both fit
 // in a block of up to 640 threads, else two passes of a block sized for the larger half.
+//
+// Chosen automatically while it has the shorter time: its threads hold the graph in registers and so issue the
+// fewest instructions per iteration, but its large blocks leave an SM idle at their barriers.  With three
+// or more blocks on an SM they cover for each other and it wins at any batch; with two or one, only up to 48 and
+// 24 shots per SM.  Measured (us, single-shot kernel | best other kernel and block size), FP32 / INT16:
+//   144 x 288, 4 and 3 blocks:  65536 shots 690 | 772 / 794 | 878
+//   192 x 400, 2 blocks:        6400 shots 338 | 351 / 373 | 391;   16384 shots 794 | 755 / 883 | 830
+//   465 x 1054, 1 block:        3200 shots 176 | 184 / 210 | 207;   6400 shots 287 | 261 / 345 | 303
+int64_t latency_limit(int per_sm) { return per_sm >= 3 ? INT64_MAX : per_sm == 2 ? 48 : 24; }
+
 int plan_latency(const qldpc_graph *const *gs, int nprob, int32_t batch, int precision, bool learned, Plan &pl,
                  bool &chosen)
 {
@@ -597,7 +608,6 @@ int plan_latency(const qldpc_graph *const *gs, int nprob, int32_t batch, int pre
     chosen = false;
     if (g0->user_kernel == QLDPC_KERNEL_BATCH || g0->user_kernel == QLDPC_KERNEL_PACKED) return QLDPC_OK;
     const bool forced = g0->user_kernel == QLDPC_KERNEL_LATENCY;
-    if (!forced && int64_t(batch) * nprob > g0->sm_count) return QLDPC_OK;
     int one = 32, two = 32;
     size_t smem = 0;
     for (int i = 0; i < nprob; ++i) {
@@ -619,29 +629,59 @@ int plan_latency(const qldpc_graph *const *gs, int nprob, int32_t batch, int pre
     const void *k = msa_kernel(precision, pl.kc);
     if (int rc = ensure_kernel_attrs(k, smem, g0->smem_optin)) return rc;
     pl.grid = batch;
-    if (forced || int64_t(batch) * nprob > g0->sm_count)
-        if (int rc = occupancy_grid(g0, k, threads, smem, nprob, batch, g0->user_blocks_per_sm, pl.grid))
-            return rc;
+    if (forced) {
+        if (int rc = occupancy_grid(g0, k, threads, smem, nprob, batch, g0->user_blocks_per_sm, pl.grid)) return rc;
+    } else if (int64_t(batch) * nprob > g0->sm_count) {   // (else every shot gets its own SM)
+        int per_sm = 0;
+        if (int rc = blocks_per_sm(k, threads, smem, per_sm)) return rc;
+        if (per_sm < 1 || shots_per_sm(g0, nprob, batch) > latency_limit(per_sm)) return QLDPC_OK;
+        if (int rc = occupancy_grid(g0, k, threads, smem, nprob, batch, per_sm, pl.grid)) return rc;
+    }
     chosen = true;
     return QLDPC_OK;
 }
 
 // Throughput path: two shots per block with their messages paired in one slot (every precision,
 // unless the graph's launch override asks for one shot per block, or the shot is learned), or one
-// shot per block.  Measured on LP-1054 at 65536 shots: FP32 31.7 M/s in pairs against 26.9, INT16
-// 31.3 against 25.5, INT8 37.7 (half-precision lanes) against 26.3.
+// shot per block.  Pairs share the graph's reads and half of the instructions, but a pair needs twice the shots
+// for the same number of busy blocks, so they start at 64 shots per SM (40 in INT8, whose pairs gain most).
+// LP-1054, one shot | two shots per block (us): FP32 6400 shots 261 | 332, 16384 shots 519 | 555 at p = 0.03 and
+// 1121 | 1072 at 0.05, 65536 shots 1727 | 1639; INT16 6400 303 | 364, 16384 592 | 585, 65536 2022 | 1781; INT8 6400
+// 283 | 285, 16384 548 | 492, 65536 1836 | 1484.
+//
+// Threads per block.  Barriers and uneven last passes cost large blocks more than their shots' shorter
+// latency gives while there are shots for many blocks: a quarter of the checks, at most 128 (65536 shots
+// in pairs, us at 64 / 96 / 128 threads: LP-1054 FP32 2164 / 1798 / 1639, the 192-check code 2477 / 2536 / 2754).  With
+// fewer shots per SM the time of the slowest one counts: 512 threads up to 4 shots per SM, 256 up to 12, 128 up
+// to 64 (rows of 9 on 1519 variables, us at 128 / 256 / 512 threads: 304 shots 149 / 126 / 126, 1000 shots 228 / 189 /
+// 212, 3200 shots 367 / 383 / 493; the 192-check code learned, 6400 shots at 64 / 128: 319 / 272).  A graph of which
+// few shots fit an SM's shared memory gets the threads that fill it, 1024 an SM (640 in pairs, whose threads need
+// more registers): 1800 checks, 4096 shots at 128 / 256 / 512 threads 716 / 507 / 440.
+int batch_threads(const qldpc_graph *const *gs, int nprob, int64_t per_sm, size_t smem, bool packed)
+{
+    int m = 1;
+    for (int i = 0; i < nprob; ++i) m = std::max(m, int(gs[i]->m));
+    const int by_shots = per_sm <= 4 ? 512 : per_sm <= 12 ? 256 : per_sm <= 64 ? 128 : std::min(128, round32((m + 3) / 4));
+    const int resident = int(std::max<size_t>(1, (gs[0]->smem_optin + 1024) / (smem + 1024)));   // blocks by shared memory
+    const int fill = (packed ? 640 : 1024) / resident / 32 * 32;
+    return std::min({packed ? kPackedMaxThreads : 1024, round32(m), std::max(by_shots, fill)});
+}
+
 int plan_batch(const qldpc_graph *const *gs, int nprob, int32_t batch, int precision, bool learned, Plan &pl)
 {
     const qldpc_graph *g0 = gs[0];
     const int word = precision == QLDPC_FP32 ? 8 : 4;   // bytes of one paired slot
+    const int64_t per_sm = shots_per_sm(g0, nprob, batch);
+    const bool forced = g0->user_kernel == QLDPC_KERNEL_PACKED;
     bool packed = !learned && g0->user_kernel != QLDPC_KERNEL_BATCH;
     for (int i = 0; i < nprob && packed; ++i)
         if (!gs[i]->dg.vslot16) {   // 16-bit slot indices: any graph whose pair of shots fits on chip
-            if (g0->user_kernel == QLDPC_KERNEL_PACKED) return QLDPC_ERR_UNSUPPORTED;
+            if (forced) return QLDPC_ERR_UNSUPPORTED;
             packed = false;
         }
-    if (packed && g0->user_kernel != QLDPC_KERNEL_PACKED) {
-        // by default only where two shots fit a block's shared memory (beside 1 KB of static shared
+    if (packed && !forced) {
+        packed = per_sm > (precision == QLDPC_INT8 ? 40 : 64);
+        // and only where two shots fit a block's shared memory (beside 1 KB of static shared
         // memory); a graph whose single shot just fits keeps one shot per block
         for (int i = 0; i < nprob; ++i)
             packed = packed && packed_layout(gs[i]->m, gs[i]->nv, gs[i]->dc_max, word).total + 1024 <= g0->smem_optin;
@@ -652,7 +692,7 @@ int plan_batch(const qldpc_graph *const *gs, int nprob, int32_t batch, int preci
                                      : shot_smem(gs[i], precision));
     pl.kc = variant(gs, nprob, false, learned);
     pl.kc.packed = packed;
-    pl.threads = g0->user_threads ? g0->user_threads : kBatchThreads;
+    pl.threads = g0->user_threads ? g0->user_threads : batch_threads(gs, nprob, per_sm, smem, packed);
     if (packed && pl.threads > kPackedMaxThreads) return QLDPC_ERR_UNSUPPORTED;
     pl.smem = smem;
     const void *k = msa_kernel(precision, pl.kc);
