@@ -33,6 +33,8 @@ struct DeviceGraph {
     const uint32_t *eslot;   // [nnz] slot j*m + i of CSR edge e
     const int32_t *layer_ptr;// [nlayers + 1] layered schedule: checks of layer l are
     const uint32_t *layer_chk;//   layer_chk[layer_ptr[l] .. layer_ptr[l+1]) (ascending)
+    const uint16_t *layer_col;// [m * layer_width] variables of the check at each place of layer_chk, rows padded to
+    int32_t layer_width;     //   whole 16-byte groups (nullptr when an index exceeds 65535)
     int32_t nlayers, max_layer;
     int32_t m, n, nnz;
     int32_t nv;              // variable lanes (n <= nv)
@@ -261,7 +263,7 @@ __host__ __device__ inline PackedLayout packed_layout(int m, int nv, int dc_max,
     return l;
 }
 
-// Layered-schedule kernels, msa_layered.cu.
+// Layered-schedule kernels, msa_layered.cu (KernelChoice::dvb = 1: the register-resident one).
 const void *msa_kernel_layered(int precision, const KernelChoice &kc);
 cudaError_t launch_msa_layered(int precision, const LaunchParams &p, const KernelChoice &kc, dim3 grid, int threads,
                                size_t smem, cudaStream_t stream);

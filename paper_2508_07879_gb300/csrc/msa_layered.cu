@@ -11,9 +11,14 @@
 // layer is one more than the largest layer of an earlier check it shares a variable with): the
 // checks of a layer run in parallel, the layers in order, and every result is bit-identical to the
 // strictly serial order.  One block per shot, persistent over the batch; per shot in shared memory:
-// Q [n] (FP32, or INT32 for the fixed-point modes), the messages r in check-major slots (j*m + i),
-// the syndrome bits.
-// One barrier per layer, then a stop-test pass over all checks (block AND).
+// Q [n] (FP32, or INT32 for the fixed-point modes), the messages r in check-major slots (j*m + place of the check
+// in the order of the layers), the syndrome bits.
+// One barrier per layer, then a stop-test pass over the checks (block AND).
+// What bounds it: the layers' barriers and shared-memory round trips, and before that the loads of the edge
+// lists, eight 4-byte ones a check and layer; in the order of the layers with 16-bit indices they are one
+// 16-byte load, and the stop test leaves a warp at its first unmet check.  LP-1054, 16384 / 65536 shots: FP32 423 / 1251
+// -> 328 / 911 us, INT16 432 / 1262 -> 385 / 1121.  (Two shots per block in pairs: 376 / 1027, 504 / 1347; they gained
+// only on the 192-check code, 588 -> 534 at 16384 shots.)
 #include <cstdint>
 
 #include <cuda_runtime.h>
@@ -24,23 +29,42 @@
 namespace qldpc {
 namespace kern {
 
-// One check of the layered schedule: Q - r_old, the min-sum update of q = clamp(Q - r_old),
-// Q = (Q - r_old) + r_new.
+// The variables of the check at place x of the layer order.
+template <int DC>
+struct LayerCols {
+    uint32_t w[(DC + 7) / 8 * 4];
+    __device__ __forceinline__ LayerCols(const DeviceGraph &g, int x)
+    {
+        const uint4 *at = reinterpret_cast<const uint4 *>(g.layer_col + size_t(x) * g.layer_width);
+#pragma unroll
+        for (int i = 0; i < (DC + 7) / 8; ++i) {
+            uint4 v = make_uint4(0, 0, 0, 0);
+            if (i == 0 || 8 * i < g.layer_width) v = __ldg(at + i);
+            w[4 * i] = v.x;
+            w[4 * i + 1] = v.y;
+            w[4 * i + 2] = v.z;
+            w[4 * i + 3] = v.w;
+        }
+    }
+    __device__ __forceinline__ uint32_t operator()(int j) const { return j & 1 ? w[j / 2] >> 16 : w[j / 2] & 0xffffu; }
+};
+
+// The check at place x of the layer order: Q - r_old, the min-sum update of q = clamp(Q - r_old),
+// Q = (Q - r_old) + r_new.  Its messages sit in slots j*M + x.
 template <class P, int DC, bool UNIFORM>
-__device__ __forceinline__ void layered_check(int c, int M, int deg, uint32_t s_bit, typename P::acc_t *__restrict__ Q,
-                                              typename P::msg_t *__restrict__ slots, const uint32_t *__restrict__ ecol,
+__device__ __forceinline__ void layered_check(const DeviceGraph &g, int x, int M, int deg, uint32_t s_bit,
+                                              typename P::acc_t *__restrict__ Q, typename P::msg_t *__restrict__ slots,
                                               const LaunchParams &p)
 {
     using acc_t = typename P::acc_t;
     using mag_t = typename P::mag_t;
+    const LayerCols<DC> col(g, x);
     acc_t qu[DC], q[DC];
-    uint32_t v[DC];
     uint32_t sx = 0;
 #pragma unroll
     for (int j = 0; j < DC; ++j) {
         if (UNIFORM || j < deg) {
-            v[j] = __ldg(ecol + size_t(j) * M + c);
-            qu[j] = P::sub(Q[v[j]], load_msg<P>(slots, uint32_t(j * M + c)));
+            qu[j] = P::sub(Q[col(j)], load_msg<P>(slots, uint32_t(j * M + x)));
             q[j] = P::clampq(qu[j]);
         }
     }
@@ -51,26 +75,38 @@ __device__ __forceinline__ void layered_check(int c, int M, int deg, uint32_t s_
     for (int j = 0; j < DC; ++j) {
         if (UNIFORM || j < deg) {
             const acc_t r = out(q[j], p);
-            Q[v[j]] = P::add(qu[j], r);
-            slots[j * M + c] = P::to_msg(r);
+            Q[col(j)] = P::add(qu[j], r);
+            slots[j * M + x] = P::to_msg(r);
         }
     }
 }
 
-// 1 iff the decisions [Q < 0] of check c's variables meet s_c.
+// 1 iff the decisions [Q < 0] of every check of this thread's warp, up to the first of its passes that finds one
+// unmet, meet the syndrome (most tests fail, and most of those in the first pass).
 template <class P, int DC, bool UNIFORM>
-__device__ __forceinline__ int check_met(int c, int M, int deg, uint32_t s_bit, const typename P::acc_t *__restrict__ Q,
-                                         const uint32_t *__restrict__ ecol)
+__device__ __forceinline__ int checks_met(const DeviceGraph &g, int tid, int T, const uint8_t *__restrict__ sb,
+                                          const typename P::acc_t *__restrict__ Q)
 {
-    uint32_t par = s_bit;
+    bool ok = true;
+    for (int x0 = 0; x0 < g.m && ok; x0 += T) {
+        const int x = x0 + tid;
+        if (x < g.m) {
+            const LayerCols<DC> col(g, x);
+            const int deg = UNIFORM ? DC : int(__ldg(g.rdeg + __ldg(g.layer_chk + x)));
+            uint32_t par = sb[x];
 #pragma unroll
-    for (int j = 0; j < DC; ++j)
-        if (UNIFORM || j < deg) par ^= P::neg(Q[__ldg(ecol + size_t(j) * M + c)]) ? 1u : 0u;
-    return par == 0;
+            for (int j = 0; j < DC; ++j)
+                if (UNIFORM || j < deg) par ^= P::neg(Q[col(j)]) ? 1u : 0u;
+            ok = par == 0;
+        }
+        ok = __all_sync(0xffffffffu, ok);
+    }
+    return ok ? 1 : 0;
 }
 
 // One shot on the shared-memory layout: Q [n] starts at the quantized priors, the messages at zero,
-// sb [m] takes the syndrome bits syn(c).  Runs the layers of every iteration with one barrier each and
+// sb [m] takes the syndrome bits syn(c) (messages and bits in the order of the layers).  Runs the layers of every
+// iteration with one barrier each and
 // the stop test after the last, and returns the iterations run (all = every check satisfied).  Ends
 // with Q final and visible to the block.
 template <class P, int DC, bool UNIFORM, class Syn>
@@ -82,32 +118,23 @@ __device__ __forceinline__ int layered_smem_shot(const DeviceGraph &g, int tid, 
     using msg_t = typename P::msg_t;
     const int M = g.m, N = g.n, L = g.nlayers;
     for (int v = tid; v < N; v += T) Q[v] = P::quantize(prior[v]);
-    for (int c = tid; c < M; c += T) {
-        sb[c] = syn(c) & 1u;
-        const int deg = UNIFORM ? DC : int(__ldg(g.rdeg + c));
-        for (int j = 0; j < deg; ++j) slots[j * M + c] = msg_t(0);
+    for (int x = tid; x < M; x += T) {
+        sb[x] = syn(int(__ldg(g.layer_chk + x))) & 1u;
+        for (int j = 0; j < g.dc_max; ++j) slots[j * M + x] = msg_t(0);
     }
     __syncthreads();
-    int ok = 1;
-    for (int c = tid; c < M; c += T)
-        ok &= check_met<P, DC, UNIFORM>(c, M, UNIFORM ? DC : int(__ldg(g.rdeg + c)), sb[c], Q, g.ecol);
-    all = __syncthreads_and(ok);
+    all = __syncthreads_and(checks_met<P, DC, UNIFORM>(g, tid, T, sb, Q));
     int k = 0;
     if (!(early && all)) {
         for (k = 1; k <= p.max_iter; ++k) {
             for (int l = 0; l < L; ++l) {
                 const int lo = __ldg(g.layer_ptr + l), hi = __ldg(g.layer_ptr + l + 1);
-                for (int i = lo + tid; i < hi; i += T) {
-                    const int c = int(__ldg(g.layer_chk + i));
-                    layered_check<P, DC, UNIFORM>(c, M, UNIFORM ? DC : int(__ldg(g.rdeg + c)), sb[c], Q, slots,
-                                                  g.ecol, p);
-                }
+                for (int x = lo + tid; x < hi; x += T)
+                    layered_check<P, DC, UNIFORM>(g, x, M, UNIFORM ? DC : int(__ldg(g.rdeg + __ldg(g.layer_chk + x))), sb[x],
+                                                  Q, slots, p);
                 __syncthreads();
             }
-            ok = 1;
-            for (int c = tid; c < M; c += T)
-                ok &= check_met<P, DC, UNIFORM>(c, M, UNIFORM ? DC : int(__ldg(g.rdeg + c)), sb[c], Q, g.ecol);
-            all = __syncthreads_and(ok);
+            all = __syncthreads_and(checks_met<P, DC, UNIFORM>(g, tid, T, sb, Q));
             if (early && all) break;
         }
         if (k > p.max_iter) k = p.max_iter;
@@ -452,21 +479,11 @@ template <class P>
 cudaError_t layered_launch(const LaunchParams &p, const KernelChoice &kc, dim3 grid, int threads, size_t smem,
                            cudaStream_t stream)
 {
-#define QLDPC_L(DCV, UNI)                                                                       \
-    if (kc.dc == DCV && kc.uniform == UNI && kc.dvb == 0) {                                     \
-        kern::msa_layered_kernel<P, DCV, UNI><<<grid, threads, smem, stream>>>(p);              \
-        return cudaGetLastError();                                                              \
-    }
-    QLDPC_LAYERED_VARIANTS(QLDPC_L)
-#undef QLDPC_L
-#define QLDPC_L(DCV, UNI)                                                                       \
-    if (kc.dc == DCV && kc.uniform == UNI && kc.dvb == 1) {                                     \
-        kern::msa_layered_reg_kernel<P, DCV, UNI, kLayeredRegMaxLayers><<<grid, threads, smem, stream>>>(p); \
-        return cudaGetLastError();                                                              \
-    }
-    QLDPC_LAYERED_REG_VARIANTS(QLDPC_L)
-#undef QLDPC_L
-    return cudaErrorInvalidValue;
+    const void *k = layered_table<P>(kc);
+    if (!k) return cudaErrorInvalidValue;
+    void *args[] = {const_cast<LaunchParams *>(&p)};
+    const cudaError_t e = cudaLaunchKernel(k, grid, dim3(unsigned(threads)), args, smem, stream);
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <class P>

@@ -277,6 +277,8 @@ struct HostLayout {
     std::vector<uint32_t> ecol;    // [dc_max * m] caller's variable of each slot, ~0 for padding
     std::vector<int32_t> layer_ptr;// [nlayers + 1] layered schedule
     std::vector<uint32_t> layer_chk;// [m] checks ordered by (layer, index)
+    std::vector<uint16_t> layer_col;// [m * layer_width] their variables (empty when n > 65535)
+    int32_t layer_width = 0;
     int32_t max_layer = 0;
     int32_t nv = 0;               // variable lanes (n + idle lanes)
     std::vector<uint16_t> vslot16;// vslot as 16-bit indices (empty when a slot index exceeds 65535)
@@ -457,6 +459,15 @@ int validate_and_layout(const int32_t *row_ptr, const int32_t *col_idx, int32_t 
     out.layer_chk.assign(size_t(m), 0u);
     std::vector<int32_t> fillp(out.layer_ptr.begin(), out.layer_ptr.end() - 1);
     for (int32_t i = 0; i < m; ++i) out.layer_chk[size_t(fillp[size_t(layer[size_t(i)])]++)] = uint32_t(i);
+    out.layer_width = (dc_max + 7) / 8 * 8;
+    if (n <= 65535) {
+        out.layer_col.assign(size_t(m) * size_t(out.layer_width), uint16_t(0));
+        for (int32_t x = 0; x < m; ++x) {
+            const int32_t i = int32_t(out.layer_chk[size_t(x)]);
+            for (int32_t e = row_ptr[i]; e < row_ptr[i + 1]; ++e)
+                out.layer_col[size_t(x) * out.layer_width + size_t(e - row_ptr[i])] = uint16_t(col_idx[e]);
+        }
+    }
     return QLDPC_OK;
 }
 
@@ -715,16 +726,21 @@ int plan_layered(const qldpc_graph *const *gs, int nprob, int32_t batch, int pre
     pl.kc = variant(gs, nprob, false, false);
     pl.kc.layered = true;
     pl.threads = std::min(1024, round32(widest));
-    // Single-shot regime (every shot gets its own SM), at most 8 layers of rows of degree <= 8 and at
-    // most 256 checks per layer: the register-resident kernel (each thread owns one check per layer; Q
-    // is the only shared array) has the lower latency.  Batches take the shared-memory kernel, whose
-    // smaller register footprint keeps more shots per SM (41.8 against 34.0 M syndromes/s, LP-1054).
-    bool reg = pl.threads <= 256 && int64_t(batch) * nprob <= g0->sm_count;
+    // Up to 40 shots per SM (80 in blocks of two warps, of which an SM holds more), with at most 8 layers of rows of degree <= 8 and at most 256 checks per layer: the
+    // register-resident kernel (each thread owns one check per layer; Q is the only shared array) has the shorter
+    // time.  Larger batches take the shared-memory kernel, whose smaller register footprint keeps more shots per SM.
+    // FP32, register | shared-memory (us): LP-1054 304 shots 55 | 66, 3200 shots 157 | 173, 6400 shots 213 | 210, 65536
+    // shots 1491 | 911; the 192-check code in layer order (64 threads) 1000 shots 127 | 160, 6400 shots 268 | 314, 16384 shots
+    // 567 | 588, 65536 1997 | 1831.
+    bool reg = pl.threads <= 256 && shots_per_sm(g0, nprob, batch) <= (pl.threads <= 64 ? 80 : 40);
     for (int i = 0; i < nprob; ++i) reg = reg && gs[i]->dg.nlayers <= 8 && gs[i]->dc_max <= 8 && gs[i]->n <= 65536;
     pl.kc.dvb = reg ? 1 : 0;
     if (reg) {
         smem = 0;
         for (int i = 0; i < nprob; ++i) smem = std::max(smem, align16(size_t(gs[i]->n) * 4));
+    } else {
+        for (int i = 0; i < nprob; ++i)   // (a shot of so many variables does not fit either)
+            if (!gs[i]->dg.layer_col) return QLDPC_ERR_UNSUPPORTED;
     }
     pl.smem = smem;
     const void *k = msa_kernel(precision, pl.kc);
@@ -960,19 +976,19 @@ int qldpc_graph_create(const int32_t *row_ptr, const int32_t *col_idx, int32_t m
     }
 
     // one device block: vslot | vdeg | rdeg | vperm | eslot | slot_edge | ecol | layer_ptr | layer_chk |
-    // shot counters | vslot16 | vlane | vchk16
-    constexpr int kArrays = 13;
+    // shot counters | vslot16 | vlane | vchk16 | layer_col
+    constexpr int kArrays = 14;
     const size_t sizes[kArrays] = {hl.vslot.size() * sizeof(uint32_t), size_t(hl.nv), size_t(m),
                                    size_t(hl.nv) * sizeof(uint32_t), hl.eslot.size() * sizeof(uint32_t),
                                    hl.slot_edge.size() * sizeof(int32_t), hl.ecol.size() * sizeof(uint32_t),
                                    hl.layer_ptr.size() * sizeof(int32_t), hl.layer_chk.size() * sizeof(uint32_t),
                                    size_t(kShotCounterSlots) * 2 * sizeof(int32_t),
                                    hl.vslot16.size() * sizeof(uint16_t), hl.vlane.size() * sizeof(uint32_t),
-                                   hl.vchk16.size() * sizeof(uint16_t)};
+                                   hl.vchk16.size() * sizeof(uint16_t), hl.layer_col.size() * sizeof(uint16_t)};
     const void *srcs[kArrays] = {hl.vslot.data(), hl.vdeg.data(), hl.rdeg.data(), hl.vorder.data(),
                                  hl.eslot.data(), hl.slot_edge.data(), hl.ecol.data(),
                                  hl.layer_ptr.data(), hl.layer_chk.data(), nullptr, hl.vslot16.data(),
-                                 hl.vlane.data(), hl.vchk16.data()};
+                                 hl.vlane.data(), hl.vchk16.data(), hl.layer_col.data()};
     size_t offs[kArrays], total = 0;
     for (int i = 0; i < kArrays; ++i) {
         offs[i] = total;
@@ -1014,6 +1030,8 @@ int qldpc_graph_create(const int32_t *row_ptr, const int32_t *col_idx, int32_t m
     g->dg.vslot16 = hl.vslot16.empty() ? nullptr : reinterpret_cast<const uint16_t *>(b + offs[10]);
     g->dg.vlane = reinterpret_cast<const uint32_t *>(b + offs[11]);
     g->dg.vchk16 = hl.vchk16.empty() ? nullptr : reinterpret_cast<const uint16_t *>(b + offs[12]);
+    g->dg.layer_col = hl.layer_col.empty() ? nullptr : reinterpret_cast<const uint16_t *>(b + offs[13]);
+    g->dg.layer_width = hl.layer_width;
     g->dg.ncls = int32_t(hl.cls_end.size());
     for (size_t c = 0; c < hl.cls_end.size(); ++c) {
         g->dg.cls_end[c] = hl.cls_end[c];

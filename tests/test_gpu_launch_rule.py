@@ -46,3 +46,50 @@ def test_lines(code, precision):
         for batch in (per_sm * sms // 2, per_sm * sms // 2 + 1):
             a, b = q.decode_pair(gz, gx, s[:batch], sx[:batch], prior, prior, **how)
             assert same(a, [t[:batch] for t in ref]) and same(b, [t[:batch] for t in ref_x]), batch
+
+
+@pytest.mark.parametrize("precision", ["fp32", "int16", "int8"])
+@pytest.mark.parametrize("code", ["lp1054", "hgp400", "bb144"])
+def test_layered_line(code, precision):
+    """40 shots per SM (80 in blocks of two warps): the register-resident kernel up to there, the shared-memory kernel
+    past it."""
+    from paper_2508_07879_gb300 import qldpc as q
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    h = CODES[code]().hz_csr
+    h = w.csr_rows(h, w.layer_order(h)) if code != "lp1054" else h
+    g = q.Graph.from_csr(h)
+    assert g.layers() <= 8
+    n = (40 if code == "lp1054" else 80) * sms
+    s = torch.from_numpy(w.syndromes(h, w.iid_x_errors(h.n, 0.04, n + 1, seed=11))).cuda()
+    prior = torch.full((h.n,), w.prior_llr(0.04), device="cuda")
+    for early in (True, False):
+        how = dict(max_iter=9, alpha=0.75, precision=precision, early_stop=early, want_post=True, layered=True)
+        past = q.decode(g, s, prior, **how)
+        assert same(q.decode(g, s[:n], prior, **how), [t[:n] for t in past])
+        assert same(q.decode(g, s[:sms + 1], prior, **how), [t[:sms + 1] for t in past])
+
+
+@pytest.mark.parametrize("precision", ["fp32", "int16", "int8"])
+@pytest.mark.parametrize("lo,hi", [(2, 8), (9, 9), (2, 15), (17, 32)])
+def test_layered_rows(lo, hi, precision):
+    """Rows of one, two and four 16-byte groups of the layered edge lists, against the oracle."""
+    import oracle
+    from paper_2508_07879_gb300 import qldpc as q
+    rng = np.random.default_rng(hi)
+    d, deg = np.zeros((37, 150), np.uint8), np.zeros(150, int)
+    for i in range(37):
+        cols = rng.choice(np.nonzero(deg < 12)[0], rng.integers(lo, hi + 1), replace=False)
+        d[i, cols] = 1
+        deg[cols] += 1
+    h = w.csr_from_dense(d)
+    s = rng.integers(0, 2, (400, h.m)).astype(np.uint8)
+    s[::4] = w.syndromes(h, w.iid_x_errors(h.n, 0.02, 100, seed=12))
+    prior = rng.normal(2, 1.5, h.n).astype(np.float32)
+    ref = oracle.msa(h.row_ptr, h.col_idx, h.m, h.n, s, prior, 6, 0.75, {"fp32": "f32", "int16": "i16", "int8": "i8"}[precision],
+                     threads=8, schedule="layered")
+    err, iters, ok, post = q.decode(q.Graph.from_csr(h), torch.from_numpy(s).cuda(), torch.from_numpy(prior).cuda(), 6,
+                                    0.75, precision, want_post=True, layered=True)
+    np.testing.assert_array_equal(err.cpu().numpy(), ref["err"])
+    np.testing.assert_array_equal(iters.cpu().numpy(), ref["iters"])
+    np.testing.assert_array_equal(ok.cpu().numpy(), ref["ok"])
+    np.testing.assert_array_equal(post.cpu().numpy() * {"fp32": 1, "int16": 256, "int8": 4}[precision], ref["post"])
