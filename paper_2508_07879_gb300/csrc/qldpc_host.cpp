@@ -887,40 +887,51 @@ int reserve_stage(qldpc_graph *g, int32_t max_batch)
 // allocation known to CUDA (cudaHostAlloc / cudaMallocHost / cudaHostRegister), else nullptr.
 // The extent comes from the driver's allocation range, so a buffer that merely starts in pinned
 // memory is never read or written by a kernel beyond that allocation.
-using PointerAttrFn = CUresult (*)(void *, CUpointer_attribute, CUdeviceptr);
+using PointerAttrsFn = CUresult (*)(unsigned int, CUpointer_attribute *, void **, CUdeviceptr);
 
-PointerAttrFn pointer_attr_fn()
+PointerAttrsFn pointer_attrs_fn()
 {
-    static PointerAttrFn fn = [] {
+    static PointerAttrsFn fn = [] {
         void *f = nullptr;
         cudaDriverEntryPointQueryResult q{};
-        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &f, 12000, cudaEnableDefault, &q) !=
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &q) !=
                 cudaSuccess ||
             q != cudaDriverEntryPointSuccess)
             f = nullptr;
-        return reinterpret_cast<PointerAttrFn>(f);
+        return reinterpret_cast<PointerAttrsFn>(f);
     }();
     return fn;
 }
 
+// (One driver call a buffer: the kind of memory, its device address and the extent of its allocation
+// together.  Memory that CUDA does not know reports no kind.)
 void *mapped_host_range(const void *p, size_t bytes)
 {
-    if (!p || bytes == 0) return nullptr;
-    cudaPointerAttributes a{};
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
+    PointerAttrsFn fn = pointer_attrs_fn();
+    if (!p || bytes == 0 || !fn) return nullptr;
+    CUpointer_attribute which[5] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                    CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE,
+                                    CU_POINTER_ATTRIBUTE_IS_MANAGED};
+    CUdeviceptr at = reinterpret_cast<CUdeviceptr>(p);
+    for (int tries = 0; tries < 2; ++tries) {
+        unsigned int type = 0, managed = 0;
+        CUdeviceptr dp = 0, start = 0;
+        size_t size = 0;
+        void *out[5] = {&type, &dp, &start, &size, &managed};
+        CUresult r = fn(5, which, out, at);
+        if (r == CUDA_ERROR_INVALID_CONTEXT) {   // a thread that has made no runtime call yet
+            cudaFree(nullptr);
+            r = fn(5, which, out, at);
+        }
+        if (r != CUDA_SUCCESS || type != CU_MEMORYTYPE_HOST || managed || !dp) return nullptr;
+        if (dp != at) {              // the extent is asked for at the device address
+            at = dp;
+            continue;
+        }
+        if (start == 0 || size == 0 || dp < start || dp - start + bytes > size) return nullptr;
+        return reinterpret_cast<void *>(dp);
     }
-    if (a.type != cudaMemoryTypeHost || !a.devicePointer) return nullptr;
-    PointerAttrFn fn = pointer_attr_fn();
-    if (!fn) return nullptr;
-    CUdeviceptr start = 0;
-    size_t size = 0;
-    const CUdeviceptr dp = reinterpret_cast<CUdeviceptr>(a.devicePointer);
-    if (fn(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, dp) != CUDA_SUCCESS) return nullptr;
-    if (fn(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, dp) != CUDA_SUCCESS) return nullptr;
-    if (start == 0 || size == 0 || dp < start || dp - start + bytes > size) return nullptr;
-    return a.devicePointer;
+    return nullptr;
 }
 
 // The graph's device copy of the prior, uploaded only when it differs from the last one (caller

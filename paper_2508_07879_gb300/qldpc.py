@@ -155,13 +155,35 @@ def check(status: int, what: str = "") -> None:
         raise QldpcError(status, what)
 
 
+_addressof = ctypes.addressof
+_c_char_at = ctypes.c_char.from_buffer
+
+
 def _np_ptr(a: np.ndarray):
-    return a.ctypes.data            # an int: ctypes passes it as the void* the signature declares
+    """Address of an array's data as an int (ctypes passes it as the void* the signature declares).  The buffer
+    protocol answers in a third of the time of ``a.ctypes.data``, which takes what it refuses (read-only or empty)."""
+    try:
+        return _addressof(_c_char_at(a))
+    except (TypeError, ValueError, BufferError):
+        return a.ctypes.data
+
+
+_torch = None       # the torch module, imported on first use (importing this module needs no torch)
+
+
+def _th():
+    global _torch
+    if _torch is None:
+        import torch
+        _torch = torch
+    return _torch
 
 
 def _dev_ptr(t, dtype, shape, name):
-    """Device pointer of a contiguous CUDA tensor of the given dtype and shape (validation only)."""
-    import torch
+    """Device pointer (an int) of a contiguous CUDA tensor of the given dtype and shape (a tuple)."""
+    torch = _torch or _th()
+    if isinstance(t, torch.Tensor) and t.is_cuda and t.dtype is dtype and t.shape == shape and t.is_contiguous():
+        return t.data_ptr()
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
     if t.dtype != dtype:
@@ -170,13 +192,20 @@ def _dev_ptr(t, dtype, shape, name):
         raise ValueError(f"{name} must have shape {tuple(shape)}, got {tuple(t.shape)}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
-def _stream_handle(stream):
-    import torch
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+def _stream_handle(stream, device=None):
+    """cudaStream_t of a torch stream, by default torch's current one (on the device of the call's tensors): as a raw
+    handle, because a Stream object for it costs more than the rest of a call's arguments."""
+    if stream is not None:
+        return stream.cuda_stream
+    torch = _torch or _th()
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return torch.cuda.current_stream().cuda_stream
+    index = device.index if device is not None else None
+    return raw(torch.cuda.current_device() if index is None else index)
 
 
 class Graph:
@@ -293,27 +322,31 @@ def decode(graph: Graph, syndromes, prior, max_iter: int, alpha: float = 0.75,
     then plain min-sum for up to ``max_iter`` iterations on shots not yet decoded.  ``layered``:
     the row-serial schedule instead of flooding.
     """
-    import torch
+    torch = _torch or _th()
     batch = int(syndromes.shape[0]) if syndromes.dim() == 2 else 0
     dev = syndromes.device
+    n = graph.n
+    u8, f32 = torch.uint8, torch.float32
     if out is None:
-        err = torch.empty((batch, graph.n), dtype=torch.uint8, device=dev)
+        err = torch.empty((batch, n), dtype=u8, device=dev)
         iters = torch.empty(batch, dtype=torch.int32, device=dev)
-        ok = torch.empty(batch, dtype=torch.uint8, device=dev)
-        post = torch.empty((batch, graph.n), dtype=torch.float32, device=dev) if want_post else None
+        ok = torch.empty(batch, dtype=u8, device=dev)
+        post = torch.empty((batch, n), dtype=f32, device=dev) if want_post else None
+        outs = (err.data_ptr(), iters.data_ptr(), ok.data_ptr(), post.data_ptr() if want_post else None)
     else:
         err, iters, ok, post = out
+        outs = None
     flags = _flags(early_stop, learned, layered)
-    check(qldpc_decode_ex(graph.handle,
-                          _dev_ptr(syndromes, torch.uint8, (batch, graph.m), "syndromes"), batch,
-                          _dev_ptr(prior, torch.float32, (graph.n,), "prior"), int(max_iter),
-                          float(alpha),
-                          _dev_ptr(err, torch.uint8, (batch, graph.n), "err"),
-                          _dev_ptr(iters, torch.int32, (batch,), "iters"),
-                          _dev_ptr(ok, torch.uint8, (batch,), "ok"),
-                          _dev_ptr(post, torch.float32, (batch, graph.n), "post") if post is not None else None,
-                          PRECISIONS[precision], flags, _stream_handle(stream)),
-          "qldpc_decode_ex")
+    syn_p = _dev_ptr(syndromes, u8, (batch, graph.m), "syndromes")
+    prior_p = _dev_ptr(prior, f32, (n,), "prior")
+    if outs is None:
+        outs = (_dev_ptr(err, u8, (batch, n), "err"), _dev_ptr(iters, torch.int32, (batch,), "iters"),
+                _dev_ptr(ok, u8, (batch,), "ok"),
+                _dev_ptr(post, f32, (batch, n), "post") if post is not None else None)
+    rc = qldpc_decode_ex(graph.handle, syn_p, batch, prior_p, int(max_iter), float(alpha), *outs, PRECISIONS[precision],
+                         flags, _stream_handle(stream, dev))
+    if rc:
+        check(rc, "qldpc_decode_ex")
     return err, iters, ok, post
 
 
@@ -340,34 +373,26 @@ def decode_pair(g_z: Graph, g_x: Graph, s_x, s_z, prior_x, prior_z, max_iter: in
                 alpha: float = 0.75, precision: str = "fp32", early_stop: bool = True,
                 want_post: bool = False, stream=None, learned: bool = False, layered: bool = False):
     """X and Z halves of a CSS syndrome round in one launch; returns two (err, iters, ok, post)."""
-    import torch
+    torch = _torch or _th()
     batch = int(s_x.shape[0])
     dev = s_x.device
-    outs = []
+    u8, f32 = torch.uint8, torch.float32
+    outs, ptrs = [], []
     for g in (g_z, g_x):
-        outs.append((torch.empty((batch, g.n), dtype=torch.uint8, device=dev),
-                     torch.empty(batch, dtype=torch.int32, device=dev),
-                     torch.empty(batch, dtype=torch.uint8, device=dev),
-                     torch.empty((batch, g.n), dtype=torch.float32, device=dev) if want_post else None))
-    (ex, ix, ox, px), (ez, iz, oz, pz) = outs
-    flags = _flags(early_stop, learned, layered)
-    check(qldpc_decode_pair(g_z.handle, g_x.handle,
-                            _dev_ptr(s_x, torch.uint8, (batch, g_z.m), "s_x"),
-                            _dev_ptr(s_z, torch.uint8, (batch, g_x.m), "s_z"), batch,
-                            _dev_ptr(prior_x, torch.float32, (g_z.n,), "prior_x"),
-                            _dev_ptr(prior_z, torch.float32, (g_x.n,), "prior_z"),
-                            int(max_iter), float(alpha),
-                            _dev_ptr(ex, torch.uint8, (batch, g_z.n), "err_x"),
-                            _dev_ptr(ez, torch.uint8, (batch, g_x.n), "err_z"),
-                            _dev_ptr(ix, torch.int32, (batch,), "iters_x"),
-                            _dev_ptr(iz, torch.int32, (batch,), "iters_z"),
-                            _dev_ptr(ox, torch.uint8, (batch,), "ok_x"),
-                            _dev_ptr(oz, torch.uint8, (batch,), "ok_z"),
-                            _dev_ptr(px, torch.float32, (batch, g_z.n), "post_x") if want_post else None,
-                            _dev_ptr(pz, torch.float32, (batch, g_x.n), "post_z") if want_post else None,
-                            PRECISIONS[precision], flags, _stream_handle(stream)),
-          "qldpc_decode_pair")
-    return (ex, ix, ox, px), (ez, iz, oz, pz)
+        o = (torch.empty((batch, g.n), dtype=u8, device=dev), torch.empty(batch, dtype=torch.int32, device=dev),
+             torch.empty(batch, dtype=u8, device=dev),
+             torch.empty((batch, g.n), dtype=f32, device=dev) if want_post else None)
+        outs.append(o)
+        ptrs.append([t.data_ptr() if t is not None else None for t in o])
+    (ex, ix, ox, px), (ez, iz, oz, pz) = ptrs
+    rc = qldpc_decode_pair(g_z.handle, g_x.handle, _dev_ptr(s_x, u8, (batch, g_z.m), "s_x"),
+                           _dev_ptr(s_z, u8, (batch, g_x.m), "s_z"), batch, _dev_ptr(prior_x, f32, (g_z.n,), "prior_x"),
+                           _dev_ptr(prior_z, f32, (g_x.n,), "prior_z"), int(max_iter), float(alpha), ex, ez, ix, iz, ox,
+                           oz, px, pz, PRECISIONS[precision], _flags(early_stop, learned, layered),
+                           _stream_handle(stream, dev))
+    if rc:
+        check(rc, "qldpc_decode_pair")
+    return outs[0], outs[1]
 
 
 def decode_host(graph: Graph, syndromes: np.ndarray, prior: np.ndarray, max_iter: int,
@@ -391,10 +416,11 @@ def decode_host(graph: Graph, syndromes: np.ndarray, prior: np.ndarray, max_iter
     else:
         err, iters, ok = out
     flags = _flags(early_stop, False, layered)
-    sh = ctypes.c_void_p(stream.cuda_stream) if stream is not None else None
-    check(qldpc_decode_host(graph.handle, _np_ptr(syn), batch, _np_ptr(pr), int(max_iter),
-                            float(alpha), _np_ptr(err), _np_ptr(iters), _np_ptr(ok),
-                            PRECISIONS[precision], flags, sh), "qldpc_decode_host")
+    rc = qldpc_decode_host(graph.handle, _np_ptr(syn), batch, _np_ptr(pr), int(max_iter), float(alpha), _np_ptr(err),
+                           _np_ptr(iters), _np_ptr(ok), PRECISIONS[precision], flags,
+                           stream.cuda_stream if stream is not None else None)
+    if rc:
+        check(rc, "qldpc_decode_host")
     return err, iters, ok
 
 
@@ -415,11 +441,12 @@ def decode_pair_host(graph_z: Graph, graph_x: Graph, s_x: np.ndarray, s_z: np.nd
         out = tuple((np.empty((batch, graph_z.n), np.uint8), np.empty(batch, np.int32), np.empty(batch, np.uint8))
                     for _ in range(2))
     (ex, ix, ox), (ez, iz, oz) = out
-    sh = ctypes.c_void_p(stream.cuda_stream) if stream is not None else None
-    check(qldpc_decode_pair_host(graph_z.handle, graph_x.handle, _np_ptr(sx), _np_ptr(sz), batch, _np_ptr(px),
-                                 _np_ptr(pz), int(max_iter), float(alpha), _np_ptr(ex), _np_ptr(ez), _np_ptr(ix),
-                                 _np_ptr(iz), _np_ptr(ox), _np_ptr(oz), PRECISIONS[precision],
-                                 _flags(early_stop, False, layered), sh), "qldpc_decode_pair_host")
+    rc = qldpc_decode_pair_host(graph_z.handle, graph_x.handle, _np_ptr(sx), _np_ptr(sz), batch, _np_ptr(px),
+                                _np_ptr(pz), int(max_iter), float(alpha), _np_ptr(ex), _np_ptr(ez), _np_ptr(ix),
+                                _np_ptr(iz), _np_ptr(ox), _np_ptr(oz), PRECISIONS[precision],
+                                _flags(early_stop, False, layered), stream.cuda_stream if stream is not None else None)
+    if rc:
+        check(rc, "qldpc_decode_pair_host")
     return out
 
 
