@@ -37,7 +37,7 @@ struct qldpc_graph {
     size_t h_stage_bytes = 0;
     std::vector<float> prior_cache;
     bool prior_valid = false;
-    // learned decoding: [learned_T][dc_max * m] slot-layout weights (qldpc_graph_set_weights)
+    // learned decoding: [learned_T][learned_stride] weights in edge groups (qldpc_graph_set_weights)
     float *d_weights = nullptr;
     int32_t learned_T = 0;
     // last training launch plan (qldpc_learned.cpp), keyed by (batch, T)

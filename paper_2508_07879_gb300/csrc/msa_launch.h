@@ -53,6 +53,19 @@ struct DeviceGraph {
     int32_t cls_deg[kMaxDegClasses];
 };
 
+// Edge groups of weights and gradients: a group's values of all checks lie one after another, so that a warp's 32 checks
+// move whole sectors with one wide access.  Training, for a compiled row degree: 2 edges where groups of 4 would leave two
+// or three places of a row's last group empty (an empty place costs a reduction).
+__host__ __device__ constexpr int train_group(int dc, bool uniform) { return uniform && (dc % 4 == 1 || dc % 4 == 2) ? 2 : 4; }
+// Place of edge j of check i among m checks.
+__host__ __device__ constexpr size_t train_edge_at(int group, int i, int j, int m)
+{
+    return (size_t(j / group) * size_t(m) + size_t(i)) * size_t(group) + size_t(j % group);
+}
+
+// Learned decoding: floats of one iteration's weights, in groups of four edges (a 16-byte load each).
+__host__ __device__ constexpr size_t learned_stride(int dc_max, int m) { return size_t((dc_max + 3) / 4 * 4) * size_t(m); }
+
 // One decoding problem: a graph and the caller's buffers for one batch.
 struct Problem {
     DeviceGraph g;
@@ -62,7 +75,7 @@ struct Problem {
     int32_t *iters;          // [batch]
     uint8_t *ok;             // [batch]
     float *post;             // [batch * n] or nullptr
-    const float *weights;    // learned decoding: [learned_iters][dc_max * m] slot-layout weights
+    const float *weights;    // learned decoding: [learned_iters][learned_stride] weights in groups of four edges
     int32_t learned_iters;   // learned iterations before the plain fallback (learned kernels only)
 };
 
@@ -176,7 +189,7 @@ constexpr unsigned long long kQueueLeave = ~0ull;
 struct ServerCode {
     DeviceGraph g;
     const float *prior;         // device [n]
-    const float *weights;       // FP32 learned decoding: [learned_iters][dc_max * m], or nullptr
+    const float *weights;       // FP32 learned decoding: [learned_iters][learned_stride], or nullptr
     int32_t learned_iters;
     unsigned char *ring;        // ring_capacity slots of slot_bytes
     int32_t slot_bytes, syn_off, err_off;
@@ -315,15 +328,6 @@ struct TrainParams {
 
 constexpr int kLossError = 0;      // BCE of sigma(-Q) against the sampled error, mean over variables
 constexpr int kLossSyndrome = 1;   // BCE of the soft syndrome against s, mean over checks
-
-// Edges of a group in the training kernels' weights and gradients, for a compiled row degree: 2 where groups of 4
-// would leave two or three places of a row's last group empty.
-__host__ __device__ constexpr int train_group(int dc, bool uniform) { return uniform && (dc % 4 == 1 || dc % 4 == 2) ? 2 : 4; }
-// Place of edge j of check i among m checks.
-__host__ __device__ constexpr size_t train_edge_at(int group, int i, int j, int m)
-{
-    return (size_t(j / group) * size_t(m) + size_t(i)) * size_t(group) + size_t(j % group);
-}
 
 struct TrainChoice {
     int dc;          // exact uniform row degree 6..8, else bucket 8/16/32

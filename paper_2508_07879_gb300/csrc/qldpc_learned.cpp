@@ -153,11 +153,12 @@ int qldpc_graph_set_weights(qldpc_graph *g, const float *weights, int32_t T)
     }
     for (float x : host)
         if (!std::isfinite(x)) return QLDPC_ERR_INVALID_ARG;
-    // slot layout [T][dc_max * m]: the weight of CSR edge e at position j of row i sits at j*m + i
-    const size_t S = size_t(g->dc_max) * size_t(g->m);
+    // edge groups: the weight of CSR edge e at position j of row i sits at train_edge_at(4, i, j, m)
+    const size_t S = learned_stride(g->dc_max, g->m);
     std::vector<uint32_t> eslot(size_t(g->nnz));
     e = cudaMemcpy(eslot.data(), g->dg.eslot, eslot.size() * sizeof(uint32_t), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_status(e);
+    for (uint32_t &x : eslot) x = uint32_t(train_edge_at(4, int(x % uint32_t(g->m)), int(x / uint32_t(g->m)), g->m));
     std::vector<float> slot(size_t(T) * S, 0.0f);
     for (int32_t t = 0; t < T; ++t)
         for (int32_t i = 0; i < g->nnz; ++i) slot[size_t(t) * S + eslot[size_t(i)]] = host[size_t(t) * g->nnz + i];

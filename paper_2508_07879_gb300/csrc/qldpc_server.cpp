@@ -314,7 +314,7 @@ int qldpc_server_create(const qldpc_graph *const *graphs, const float *const *pr
         prior_off[c] = dev_bytes;
         dev_bytes += align16(size_t(s->n[c]) * sizeof(float));
         const qldpc_graph *g = graphs[c];
-        w_bytes[c] = (learned && g->d_weights) ? size_t(g->learned_T) * g->dc_max * g->m * sizeof(float) : 0;
+        w_bytes[c] = (learned && g->d_weights) ? size_t(g->learned_T) * learned_stride(g->dc_max, g->m) * sizeof(float) : 0;
         w_off[c] = dev_bytes;
         dev_bytes += align16(w_bytes[c]);
     }

@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(kLatencyMaxThreads, 1) msa_server_kernel(const
             slots = reinterpret_cast<msg_t *>(smem + latency_layout(M, sc.g.dc_max, int(sizeof(msg_t))).slot_off);
             weights = LEARNED ? sc.weights : nullptr;
             learned_iters = sc.learned_iters;
-            wstride = size_t(sc.g.dc_max) * M;
+            wstride = learned_stride(sc.g.dc_max, M);
             udc = sc.udc;
             wc.load(sc, tid, T);
         }

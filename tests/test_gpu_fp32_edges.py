@@ -52,3 +52,27 @@ def test_minima(graph, prior):
             np.testing.assert_array_equal(err.cpu().numpy(), ref["err"])
             np.testing.assert_array_equal(ok.cpu().numpy(), ref["ok"])
         g.set_launch("auto")
+
+
+@pytest.mark.parametrize("kernel", ["batch", "latency"])
+@pytest.mark.parametrize("graph", list(GRAPHS))
+def test_learned_rows(graph, kernel):
+    """Learned weights reach their edges for every row form (groups of four edges, the last one not always full)."""
+    from paper_2508_07879_gb300 import qldpc as q
+    h = GRAPHS[graph]()
+    rng = np.random.default_rng(len(graph))
+    s = rng.integers(0, 2, (35, h.m)).astype(np.uint8)
+    gamma = rng.uniform(0.5, 3.0, h.n).astype(np.float32)
+    weights = rng.uniform(0.3, 1.0, (3, h.nnz)).astype(np.float32)
+    ref = oracle.nms_decode(h.row_ptr, h.col_idx, h.m, h.n, s, gamma, weights, 3, 0.75, threads=4)
+    g = q.Graph.from_csr(h)
+    g.set_weights(weights)
+    try:
+        g.set_launch(kernel)
+    except q.QldpcError:      # (the single-shot kernel does not hold every graph)
+        assert kernel == "latency"
+        return
+    got = q.decode(g, torch.from_numpy(s).cuda(), torch.from_numpy(gamma).cuda(), 3, 0.75, learned=True,
+                   want_post=True)
+    for name, t in zip(("err", "iters", "ok", "post"), got):
+        np.testing.assert_array_equal(t.cpu().numpy(), ref[name], err_msg=name)
