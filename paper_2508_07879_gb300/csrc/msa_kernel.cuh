@@ -150,6 +150,12 @@ struct WideSlots<IFix<MSG, FRAC, LIM>> {
     using type = IFix<int32_t, FRAC, LIM>;
 };
 
+template <class T>
+__device__ __forceinline__ T *at_bytes(T *base, uint32_t offset)
+{
+    return reinterpret_cast<T *>(reinterpret_cast<unsigned char *>(base) + offset);
+}
+
 template <class P>
 __device__ __forceinline__ typename P::acc_t load_msg(const typename P::msg_t *s, uint32_t i)
 {
@@ -395,8 +401,8 @@ __device__ __forceinline__ int check_step(int c, int M, int deg, uint32_t pw, bo
 // + ... + r_{k-1}.  Stores every q_k, flips the parity bit of its checks when the decision
 // [Q < 0] differs from `prev`, and returns Q.
 // ---------------------------------------------------------------------------------------------
-// TRACK = false (training forward): no decision tracking, parity may be null.
-template <class P, int D, bool TRACK = true>
+// BYTES: sl holds byte offsets into slots instead of slot indices (lane_slots).
+template <class P, int D, bool BYTES = false>
 __device__ __forceinline__ typename P::acc_t var_step_exact(const uint32_t *sl, const CheckOf &ck, typename P::acc_t gamma,
                                                             bool prev, typename P::msg_t *__restrict__ slots,
                                                             uint32_t *__restrict__ parity)
@@ -407,7 +413,7 @@ __device__ __forceinline__ typename P::acc_t var_step_exact(const uint32_t *sl, 
     } else {
         acc_t r[D];
 #pragma unroll
-        for (int k = 0; k < D; ++k) r[k] = load_msg<P>(slots, sl[k]);
+        for (int k = 0; k < D; ++k) r[k] = typename P::acc_t(BYTES ? *at_bytes(slots, sl[k]) : slots[sl[k]]);
         acc_t pre[D + 1];
         pre[0] = gamma;
 #pragma unroll
@@ -418,11 +424,11 @@ __device__ __forceinline__ typename P::acc_t var_step_exact(const uint32_t *sl, 
             acc_t q = pre[k];
 #pragma unroll
             for (int i = k + 1; i < D; ++i) q = P::add(q, r[i]);
-            slots[sl[k]] = P::to_msg(q);
+            (BYTES ? *at_bytes(slots, sl[k]) : slots[sl[k]]) = P::to_msg(q);
         }
-        if (TRACK && P::neg(Q) != prev) {
+        if (P::neg(Q) != prev) {
 #pragma unroll
-            for (int k = 0; k < D; ++k) flip_check(parity, ck(sl[k]));
+            for (int k = 0; k < D; ++k) flip_check(parity, ck(BYTES ? sl[k] / sizeof(typename P::msg_t) : sl[k]));
         }
         return Q;
     }
@@ -457,13 +463,39 @@ __device__ __forceinline__ void for_lanes(const DeviceGraph &G, int tid, int T, 
     }
 }
 
-// The edge list of lane u from the 16-bit lists, or from the 32-bit ones on a graph with more slots than they
-// index (no such graph fits a block in FP32).
-template <int D, bool WIDE>
-__device__ __forceinline__ void lane_edges(const DeviceGraph &g, int u, uint32_t (&e)[D > 0 ? D : 1])
+// The edge slots of lane u as byte offsets into words of WORD bytes, from the 16-bit lists (vslot16): four slots come with
+// one load, and one two-way dot product takes a slot out of its register and scales it.  The variable steps are short of
+// load instructions (a slot a load: 16384 learned shots of LP-1054 550 -> 531 us, 8191 of its 465 x 1519 data-syndrome
+// graph 746 -> 714, 4096 in INT16 212 -> 204; the paired FP32 kernel, which waits on its 8-byte slots, 3631 -> 3619).
+template <int D, int WORD>
+__device__ __forceinline__ void lane_slots(const uint16_t *__restrict__ list, int NV, int u, uint32_t (&o)[D > 0 ? D : 1])
 {
 #pragma unroll
-    for (int k = 0; k < D; ++k) e[k] = WIDE ? __ldg(g.vslot + size_t(k) * g.nv + u) : uint32_t(__ldg(g.vslot16 + k * g.nv + u));
+    for (int k = 0; k < D; k += 4) {
+        const uint16_t *at = list + (size_t(k / 4) * NV + u) * 4;
+        uint2 v = make_uint2(0u, 0u);
+        if (D - k > 2)
+            v = __ldg(reinterpret_cast<const uint2 *>(at));
+        else if (D - k == 2)
+            v.x = __ldg(reinterpret_cast<const unsigned *>(at));
+        else
+            v.x = __ldg(at);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (k + i < D) o[k + i] = __dp2a_lo(i < 2 ? v.x : v.y, unsigned(i & 1 ? WORD << 8 : WORD), 0u);
+    }
+}
+
+// The same from the 32-bit lists on a graph with more slots than 16 bits index (no such graph fits a block in FP32).
+template <int D, int WORD, bool WIDE>
+__device__ __forceinline__ void lane_edges(const DeviceGraph &g, int u, uint32_t (&o)[D > 0 ? D : 1])
+{
+    if constexpr (WIDE) {
+#pragma unroll
+        for (int k = 0; k < D; ++k) o[k] = __ldg(g.vslot + size_t(k) * g.nv + u) * WORD;
+    } else {
+        lane_slots<D, WORD>(g.vslot16, g.nv, u, o);
+    }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -482,13 +514,13 @@ __device__ __forceinline__ void batch_init_shot(const DeviceGraph &g, const uint
     for_lanes<DV>(g, tid, T, [&](auto deg, int u) {
         constexpr int D = decltype(deg)::value;
         uint32_t e[D > 0 ? D : 1];
-        lane_edges<D, WIDE>(g, u, e);
+        lane_edges<D, sizeof(typename P::msg_t), WIDE>(g, u, e);
         const typename P::acc_t x = gam[u];
         const bool d = P::neg(x);
 #pragma unroll
         for (int k = 0; k < D; ++k) {
-            slots[e[k]] = P::to_msg(x);
-            if (d) flip_check(parity, ck(e[k]));
+            *at_bytes(slots, e[k]) = P::to_msg(x);
+            if (d) flip_check(parity, ck(e[k] / sizeof(typename P::msg_t)));
         }
         Qs[u] = x;
     });
@@ -582,8 +614,8 @@ __device__ __forceinline__ void batch_decode(const LaunchParams &p)
             for_lanes<DV>(G, tid, T, [&](auto deg, int u) {
                 constexpr int D = decltype(deg)::value;
                 uint32_t e[D > 0 ? D : 1];
-                lane_edges<D, WIDE>(G, u, e);
-                Qs[u] = var_step_exact<P, D>(e, ck, gam[u], P::neg(Qs[u]), slots, parity);
+                lane_edges<D, sizeof(msg_t), WIDE>(G, u, e);
+                Qs[u] = var_step_exact<P, D, true>(e, ck, gam[u], P::neg(Qs[u]), slots, parity);
             });
             __syncthreads();
             ++k;

@@ -41,13 +41,14 @@ struct DeviceGraph {
     uint32_t m_magic;        // floor(slot / m) = umulhi(slot, m_magic) >> m_shift for every slot
     int32_t m_shift;
     int32_t dc_max, dv_max;  // largest row / column degree
-    // The same slot lists as 16-bit indices (nullptr when a slot index exceeds 65535), and the lanes'
+    // The same slot lists as 16-bit indices, four of a lane's slots side by side: its k-th slot at
+    // vslot16[((k / 4) * nv + u) * 4 + k % 4] (nullptr when a slot index exceeds 65535), and the lanes'
     // degree classes: lanes [cls_end[c-1], cls_end[c]) (cls_end[-1] = 0) all have degree cls_deg[c],
     // c < ncls.  The two-shots-per-block kernel walks the classes with the degree known at compile
     // time instead of reading vdeg per lane.
     const uint16_t *vslot16;
     const uint32_t *vlane;   // [n] lane of each variable (the inverse of vperm on the real lanes)
-    const uint16_t *vchk16;  // [dv_max * nv] the check of each vslot16 entry (slot mod m), with vslot16
+    const uint16_t *vchk16;  // [dv_max * nv] the check of each vslot entry (slot mod m), with vslot16
     int32_t ncls;
     int32_t cls_end[kMaxDegClasses];
     int32_t cls_deg[kMaxDegClasses];

@@ -192,10 +192,9 @@ __device__ __forceinline__ int2 var_step_x2(int u, int NV, const uint16_t *__res
         return make_int2(gamma, gamma);
     } else {
         uint32_t e[D], r[D];
+        lane_slots<D, 4>(vslot, NV, u, e);
 #pragma unroll
-        for (int k = 0; k < D; ++k) e[k] = __ldg(vslot + k * NV + u);
-#pragma unroll
-        for (int k = 0; k < D; ++k) r[k] = MASK ? slots[e[k]] & keep : slots[e[k]];
+        for (int k = 0; k < D; ++k) r[k] = MASK ? *at_bytes(slots, e[k]) & keep : *at_bytes(slots, e[k]);
         int32_t Q0 = gamma, Q1 = gamma;
 #pragma unroll
         for (int k = 0; k < D; ++k) {
@@ -203,7 +202,7 @@ __device__ __forceinline__ int2 var_step_x2(int u, int NV, const uint16_t *__res
             Q1 += lane1(r[k]);
         }
 #pragma unroll
-        for (int k = 0; k < D; ++k) slots[e[k]] = clamp_pair<P>(Q0 - lane0(r[k]), Q1 - lane1(r[k]));
+        for (int k = 0; k < D; ++k) *at_bytes(slots, e[k]) = clamp_pair<P>(Q0 - lane0(r[k]), Q1 - lane1(r[k]));
         const uint32_t flip = (uint32_t(Q0 ^ Qold.x) >> 31) | ((uint32_t(Q1 ^ Qold.y) >> 31) << 16);
         if (flip) {
 #pragma unroll
@@ -281,11 +280,10 @@ __device__ __forceinline__ float2 var_step_f32x2(int u, int NV, const CheckOf &c
         const uint32_t k0 = (act & 1u) ? 0xffffffffu : 0u, k1 = (act & 2u) ? 0xffffffffu : 0u;
         uint32_t e[D];
         float2 r[D];
-#pragma unroll
-        for (int k = 0; k < D; ++k) e[k] = __ldg(vslot + k * NV + u);
+        lane_slots<D, 8>(vslot, NV, u, e);
 #pragma unroll
         for (int k = 0; k < D; ++k) {
-            const float2 v = slots[e[k]];        // a lane that restarts takes r = +0: Q = q = gamma
+            const float2 v = *at_bytes(slots, e[k]);        // a lane that restarts takes r = +0: Q = q = gamma
             r[k] = MASK ? make_float2(__uint_as_float(__float_as_uint(v.x) & k0), __uint_as_float(__float_as_uint(v.y) & k1))
                         : v;
         }
@@ -299,7 +297,7 @@ __device__ __forceinline__ float2 var_step_f32x2(int u, int NV, const CheckOf &c
             float2 q = pre[k];
 #pragma unroll
             for (int i = k + 1; i < D; ++i) q = add2_rn(q, r[i]);
-            slots[e[k]] = q;
+            *at_bytes(slots, e[k]) = q;
         }
         // the lanes whose decision [Q < 0] changed: the sign bits differ (no Q is -0, and the only NaN
         // the arithmetic can form, inf - inf, is the positive canonical one)
@@ -307,7 +305,7 @@ __device__ __forceinline__ float2 var_step_f32x2(int u, int NV, const CheckOf &c
                               (((__float_as_uint(Q.y) ^ __float_as_uint(Qold.y)) >> 15) & 0x00010000u);
         if (flip) {
 #pragma unroll
-            for (int k = 0; k < D; ++k) atomicXor(parity + ck(e[k]), flip);
+            for (int k = 0; k < D; ++k) atomicXor(parity + ck(e[k] / 8), flip);
         }
         return Q;
     }
@@ -476,10 +474,9 @@ __device__ __forceinline__ uint32_t var_step_h8(int u, int NV, const uint16_t *_
         return gamma;
     } else {
         uint32_t e[D], r[D];
+        lane_slots<D, 4>(vslot, NV, u, e);
 #pragma unroll
-        for (int k = 0; k < D; ++k) e[k] = __ldg(vslot + k * NV + u);
-#pragma unroll
-        for (int k = 0; k < D; ++k) r[k] = MASK ? slots[e[k]] & keep : slots[e[k]];   // restart: r = +0
+        for (int k = 0; k < D; ++k) r[k] = MASK ? *at_bytes(slots, e[k]) & keep : *at_bytes(slots, e[k]);   // restart: r = +0
         uint32_t pre[D + 1];
         pre[0] = gamma;
 #pragma unroll
@@ -490,7 +487,7 @@ __device__ __forceinline__ uint32_t var_step_h8(int u, int NV, const uint16_t *_
             uint32_t q = pre[k];
 #pragma unroll
             for (int i = k + 1; i < D; ++i) q = h2_add(q, r[i]);
-            slots[e[k]] = h2_max(h2_min(q, kH2Lim), kH2NegLim);
+            *at_bytes(slots, e[k]) = h2_max(h2_min(q, kH2Lim), kH2NegLim);
         }
         const uint32_t flip = ((Q ^ Qold) >> 15) & 0x00010001u;   // lane decisions that changed (bits 0 / 16)
         if (flip) {

@@ -373,8 +373,10 @@ __global__ void __launch_bounds__(kTrainThreads, DC <= 8 ? 3 : 1) nms_forward_ke
         const float g = F32::quantize(lane_prior(G, p.prior, u));
         gam[u] = g;
         if constexpr (!SYN) y[u] = lane_targets<L>(G, p.target, shot, u);
+        uint32_t e[D > 0 ? D : 1];
+        lane_slots<D, sizeof(word)>(G.vslot16, NV, u, e);
 #pragma unroll
-        for (int i = 0; i < D; ++i) slots[__ldg(G.vslot16 + i * NV + u)] = V::all(g);
+        for (int i = 0; i < D; ++i) *at_bytes(slots, e[i]) = V::all(g);
     });
     __syncthreads();
     float acc[L];
@@ -408,10 +410,9 @@ __global__ void __launch_bounds__(kTrainThreads, DC <= 8 ? 3 : 1) nms_forward_ke
             constexpr int D = decltype(deg)::value;
             uint32_t e[D > 0 ? D : 1];
             word r[D > 0 ? D : 1], pre[D + 1];
+            lane_slots<D, sizeof(word)>(G.vslot16, NV, u, e);
 #pragma unroll
-            for (int i = 0; i < D; ++i) e[i] = __ldg(G.vslot16 + i * NV + u);
-#pragma unroll
-            for (int i = 0; i < D; ++i) r[i] = slots[e[i]];
+            for (int i = 0; i < D; ++i) r[i] = *at_bytes(slots, e[i]);
             pre[0] = V::all(gam[u]);
 #pragma unroll
             for (int i = 0; i < D; ++i) pre[i + 1] = V::add(pre[i], r[i]);
@@ -421,14 +422,14 @@ __global__ void __launch_bounds__(kTrainThreads, DC <= 8 ? 3 : 1) nms_forward_ke
                 word q = pre[i];
 #pragma unroll
                 for (int h = i + 1; h < D; ++h) q = V::add(q, r[h]);
-                slots[e[i]] = q;
+                *at_bytes(slots, e[i]) = q;
             }
             if constexpr (SYN) {
                 word code;
 #pragma unroll
                 for (int l = 0; l < L; ++l) V::set(code, l, soft_code(V::get(Q, l)));
 #pragma unroll
-                for (int i = 0; i < D; ++i) ts[e[i]] = code;
+                for (int i = 0; i < D; ++i) *at_bytes(ts, e[i]) = code;
             } else if (y[u] != kIdleLane) {
 #pragma unroll
                 for (int l = 0; l < L; ++l) {
@@ -554,16 +555,15 @@ __global__ void __launch_bounds__(kTrainThreads, DC <= 8 ? 3 : 1) nms_backward_k
             for_lanes<DV>(G, tid, T, [&](auto deg, int u) {
                 constexpr int D = decltype(deg)::value;
                 uint32_t e[D > 0 ? D : 1];
-#pragma unroll
-                for (int i = 0; i < D; ++i) e[i] = __ldg(G.vslot16 + i * NV + u);
+                lane_slots<D, sizeof(word)>(G.vslot16, NV, u, e);
                 word Q = V::all(gam[u]), code;
 #pragma unroll
-                for (int i = 0; i < D; ++i) Q = V::add(Q, rs[e[i]]);
+                for (int i = 0; i < D; ++i) Q = V::add(Q, *at_bytes(rs, e[i]));
 #pragma unroll
                 for (int l = 0; l < L; ++l) V::set(code, l, soft_code(V::get(Q, l)));
                 ucode[u] = code;
 #pragma unroll
-                for (int i = 0; i < D; ++i) ts[e[i]] = code;
+                for (int i = 0; i < D; ++i) *at_bytes(ts, e[i]) = code;
             });
             __syncthreads();
             for (int c = tid; c < M; c += T)
@@ -575,17 +575,16 @@ __global__ void __launch_bounds__(kTrainThreads, DC <= 8 ? 3 : 1) nms_backward_k
             constexpr int D = decltype(deg)::value;
             uint32_t e[D > 0 ? D : 1];
             word g[D > 0 ? D : 1], sum = V::all(0.0f), gQ;
-#pragma unroll
-            for (int i = 0; i < D; ++i) e[i] = __ldg(G.vslot16 + i * NV + u);
+            lane_slots<D, sizeof(word)>(G.vslot16, NV, u, e);
 #pragma unroll
             for (int i = 0; i < D; ++i) {
-                g[i] = gs[e[i]];
+                g[i] = *at_bytes(gs, e[i]);
                 sum = V::add(sum, g[i]);
             }
             if constexpr (SYN) {
                 word H = V::all(0.0f), slope;
 #pragma unroll
-                for (int i = 0; i < D; ++i) H = V::add(H, ts[e[i]]);
+                for (int i = 0; i < D; ++i) H = V::add(H, *at_bytes(ts, e[i]));
                 const word code = ucode[u];
 #pragma unroll
                 for (int l = 0; l < L; ++l) V::set(slope, l, code_slope(V::get(code, l)));
@@ -593,13 +592,13 @@ __global__ void __launch_bounds__(kTrainThreads, DC <= 8 ? 3 : 1) nms_backward_k
             } else {
                 word Q = V::all(gam[u]);
 #pragma unroll
-                for (int i = 0; i < D; ++i) Q = V::add(Q, rs[e[i]]);
+                for (int i = 0; i < D; ++i) Q = V::add(Q, *at_bytes(rs, e[i]));
 #pragma unroll
                 for (int l = 0; l < L; ++l)
                     V::set(gQ, l, V::get(gk, l) * (float((y[u] >> l) & 1u) - sigmoid(-V::get(Q, l))));
             }
 #pragma unroll
-            for (int i = 0; i < D; ++i) gs[e[i]] = V::add(gQ, V::sub(sum, g[i]));
+            for (int i = 0; i < D; ++i) *at_bytes(gs, e[i]) = V::add(gQ, V::sub(sum, g[i]));
         });
         __syncthreads();
         // check side: weight gradient, dL/dq of iteration k, and r of iteration k-1

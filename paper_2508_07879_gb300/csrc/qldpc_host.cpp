@@ -281,8 +281,8 @@ struct HostLayout {
     int32_t layer_width = 0;
     int32_t max_layer = 0;
     int32_t nv = 0;               // variable lanes (n + idle lanes)
-    std::vector<uint16_t> vslot16;// vslot as 16-bit indices (empty when a slot index exceeds 65535)
-    std::vector<uint16_t> vchk16; // the check i = slot mod m of each vslot16 entry (same layout)
+    std::vector<uint16_t> vslot16;// [dv_max / 4 rounded up][nv][4] as 16-bit indices (empty when one exceeds 65535)
+    std::vector<uint16_t> vchk16; // the check i = slot mod m of each vslot entry (same layout)
     std::vector<int32_t> cls_end, cls_deg;   // runs of equal lane degree
     uint32_t m_magic = 0;         // slot / m = umulhi(slot, m_magic) >> m_shift
     int32_t m_shift = 0;
@@ -407,7 +407,11 @@ int validate_and_layout(const int32_t *row_ptr, const int32_t *col_idx, int32_t 
         }
     }
     if (S + size_t(kScratch) <= 65536) {
-        out.vslot16.assign(out.vslot.begin(), out.vslot.end());
+        out.vslot16.assign((out.vslot.size() / nv + 3) / 4 * 4 * nv, uint16_t(0));
+        for (size_t t = 0; t < out.vslot.size(); ++t) {
+            const size_t k = t / nv, u = t % nv;
+            out.vslot16[(k / 4 * nv + u) * 4 + k % 4] = uint16_t(out.vslot[t]);
+        }
         out.vchk16.resize(out.vslot.size());
         for (size_t t = 0; t < out.vslot.size(); ++t) out.vchk16[t] = uint16_t(out.vslot[t] % uint32_t(m));
     }
