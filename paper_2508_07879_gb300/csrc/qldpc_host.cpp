@@ -659,10 +659,13 @@ int plan_latency(const qldpc_graph *const *gs, int nprob, int32_t batch, int pre
 // Throughput path: two shots per block with their messages paired in one slot (every precision,
 // unless the graph's launch override asks for one shot per block, or the shot is learned), or one
 // shot per block.  Pairs share the graph's reads and half of the instructions, but a pair needs twice the shots
-// for the same number of busy blocks, so they start at 64 shots per SM (40 in INT8, whose pairs gain most).
-// LP-1054, one shot | two shots per block (us): FP32 6400 shots 261 | 332, 16384 shots 519 | 555 at p = 0.03 and
-// 1121 | 1072 at 0.05, 65536 shots 1727 | 1639; INT16 6400 303 | 364, 16384 592 | 585, 65536 2022 | 1781; INT8 6400
-// 283 | 285, 16384 548 | 492, 65536 1836 | 1484.
+// for the same number of busy blocks, spends more on each new shot and reads its slots 8 bytes at a time in FP32.
+// Long decodes gain and short ones lose.  FP32: the line lies where the times summed over physical error rates 0.01,
+// 0.02 .. 0.05 cross, 320 shots per SM (those sums in us, one shot | two shots per block, LP-1054 and the 192-check code:
+// 20000 shots 3268 | 3454 and 2355 | 2705, 49152 shots 7330 | 7326 and 5141 | 5223, 65536 shots 9618 | 9499 and 6697 |
+// 6668; at the ends 16384 shots at 0.01 248 | 291 and 157 | 258, 65536 shots at 0.05 3838 | 3617 and 2565 | 2398).
+// INT16 and INT8: where the noisiest decodes cross, 80 and 40 shots per SM (LP-1054 at 0.05: INT16 12000 shots 956 |
+// 938, 16384 shots 1258 | 1182; INT8 8192 shots 662 | 588).
 //
 // Threads per block.  Barriers and uneven last passes cost large blocks more than their shots' shorter
 // latency gives while there are shots for many blocks: a quarter of the checks, at most 128 (65536 shots
@@ -695,7 +698,7 @@ int plan_batch(const qldpc_graph *const *gs, int nprob, int32_t batch, int preci
             packed = false;
         }
     if (packed && !forced) {
-        packed = per_sm > (precision == QLDPC_INT8 ? 40 : 64);
+        packed = per_sm > (precision == QLDPC_INT8 ? 40 : precision == QLDPC_INT16 ? 80 : 320);
         // and only where two shots fit a block's shared memory (beside 1 KB of static shared
         // memory); a graph whose single shot just fits keeps one shot per block
         for (int i = 0; i < nprob; ++i)

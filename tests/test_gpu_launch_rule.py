@@ -93,3 +93,22 @@ def test_layered_rows(lo, hi, precision):
     np.testing.assert_array_equal(iters.cpu().numpy(), ref["iters"])
     np.testing.assert_array_equal(ok.cpu().numpy(), ref["ok"])
     np.testing.assert_array_equal(post.cpu().numpy() * {"fp32": 1, "int16": 256, "int8": 4}[precision], ref["post"])
+
+
+@pytest.mark.parametrize("precision,per_sm", [("fp32", 320), ("int16", 80), ("int8", 40)])
+@pytest.mark.parametrize("code", ["hgp400", "lp1054"])
+def test_pair_line(code, precision, per_sm):
+    """One shot per block up to the line, two past it (an odd batch: the last block has one)."""
+    from paper_2508_07879_gb300 import qldpc as q
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    h = CODES[code]().hz_csr
+    g = q.Graph.from_csr(h)
+    most = per_sm * sms + 1
+    s = torch.from_numpy(w.syndromes(h, w.iid_x_errors(h.n, 0.04, most, seed=11))).cuda()
+    prior = torch.full((h.n,), w.prior_llr(0.04), device="cuda")
+    how = dict(max_iter=8, alpha=0.75, precision=precision, want_post=True)
+    g.set_launch("batch", 128)
+    ref = q.decode(g, s, prior, **how)
+    g.set_launch("auto")
+    for batch in (most - 1, most - most % 2 - 1, most):
+        assert same(q.decode(g, s[:batch], prior, **how), [t[:batch] for t in ref]), batch
