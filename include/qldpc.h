@@ -161,13 +161,14 @@ QLDPC_API int qldpc_graph_footprint(const qldpc_graph *g, int32_t precision, int
 
 /* Kernels (qldpc_graph_set_launch). */
 enum {
-    QLDPC_KERNEL_AUTO = 0,      /* latency kernel when every shot gets its own SM, else the packed
-                                   kernel where two shots fit a block's shared memory (learned
-                                   decoding: the batch kernel) */
+    QLDPC_KERNEL_AUTO = 0,      /* by shots per SM: the latency kernel for single shots and moderate
+                                   batches (any batch of a small code), then the batch kernel, and the
+                                   packed kernel for the largest batches where two shots fit a block's
+                                   shared memory (learned decoding: never the packed kernel) */
     QLDPC_KERNEL_BATCH = 1,     /* throughput kernel: one shot per block, thread per check / per
                                    variable, persistent blocks */
-    QLDPC_KERNEL_LATENCY = 2,   /* single-shot kernel: per-thread state in registers, one block per
-                                   shot; needs m <= 2*threads and n <= 2*threads, threads <= 640 */
+    QLDPC_KERNEL_LATENCY = 2,   /* per-thread state in registers, one shot per block at a time;
+                                   needs m <= 2*threads and n <= 2*threads, threads <= 640 */
     QLDPC_KERNEL_PACKED = 3     /* throughput kernel with two shots per block, their messages paired
                                    in one slot per edge (a float2 in FP32, two 16-bit integer lanes in
                                    INT16, two half-precision lanes holding the exact INT8 integers up

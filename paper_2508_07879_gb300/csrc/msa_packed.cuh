@@ -1,5 +1,5 @@
-// Two shots per block, their messages paired in one slot per edge: the throughput kernel of every
-// precision.
+// Two shots per block, their messages paired in one slot per edge: the kernel of the largest batches in every
+// precision (from where on: plan_batch in qldpc_host.cpp).
 //
 // Algorithm 1 (Sec. 2 of arXiv 2508.07879) with the arithmetic of the precision policies of
 // msa_kernel.cuh, but every shared-memory slot holds the same edge's message of two shots: lane 0

@@ -22,13 +22,14 @@
 // L = 1 or 2 shots per block.  Two shots share every weight, edge list and prior, their messages sit in one
 // 8-byte slot per edge (as in the two-shots-per-block decoder), their sums and products are packed FP32
 // operations.  Weights and their gradient lie in groups of four edges (two where a row's length asks for it), so a
-// check moves four of them per instruction and a warp whole sectors.  Each shot's gradient is added by itself: adding the pair first halves the
-// reductions but changes the order of the sum over shots, whose rounding is the largest error of a gradient.
+// check moves four of them per instruction and a warp whole sectors; a lane's edge slots come four to a load.  Each
+// shot's gradient is added by itself: adding the pair first halves the reductions but changes the order of the sum over
+// shots, whose rounding is the largest error of a gradient.
 // What bounds both kernels is instruction issue and the latency of short chains between barriers, not
 // memory: the recorded state (16 bytes per check, iteration and shot, written once and read from L2 after
 // a prefetch) and the gradient's reductions are the only traffic.
-// LP-1054, 4096 shots, T = 20, syndrome loss: forward 1097 -> 528 us, backward 2664 -> 872 us
-// (error loss 784 -> 619 and 1687 -> 679).
+// LP-1054, 4096 shots, T = 20, syndrome loss: forward 1097 -> 516 us, backward 2664 -> 830 us
+// (error loss 784 -> 607 and 1687 -> 685).
 #pragma once
 
 #include <cstdint>
