@@ -367,7 +367,7 @@ cudaError_t launch_logical(const LogicalPlan &pl, const uint8_t *logicals, int32
 
 // Shared memory of a training block of `shots` shots (n = variable lanes).  Forward: the messages, the codes per
 // edge (syndrome loss), the priors, targets and syndrome bits.  Backward: the gradient slots, the r slots
-// (the syndrome loss's codes overwrite them in place), the code per lane (syndrome loss), and the rest.
+// (the syndrome loss's codes overwrite them in place), Q per lane (syndrome loss), and the rest.
 struct TrainLayout {
     size_t slot_off, r_off, q_off, g_off, y_off, s_off, total;
 };

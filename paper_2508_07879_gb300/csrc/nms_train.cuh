@@ -17,19 +17,25 @@
 //                          dL/dq_{m,idx2} = dL/dr_{m,idx1} w sign * sign(q_idx2)     (all other q: 0)
 //                        Weight gradients are added into one L2-resident buffer with global
 //                        reductions, so the order of the sum over shots follows the schedule: the
-//                        last bits of a gradient can differ between calls.
+//                        last bits of a gradient can differ between calls.  The next step can make
+//                        much more of them: min-sum's gradient jumps where a minimum changes place, so a
+//                        weight that is off in its last bit moves one shot's whole share.  LP-1054, 4096
+//                        shots, T = 20: two runs of a step differ by 5e-7 of the gradient's norm, 30 of
+//                        its 74400 weights then differ in the last bit, and after one more step the two
+//                        gradients are more than 2e-5 apart for 3 of 10 inputs (up to 4e-3).
 //
 // L = 1 or 2 shots per block.  Two shots share every weight, edge list and prior, their messages sit in one
 // 8-byte slot per edge (as in the two-shots-per-block decoder), their sums and products are packed FP32
 // operations.  Weights and their gradient lie in groups of four edges (two where a row's length asks for it), so a
 // check moves four of them per instruction and a warp whole sectors; a lane's edge slots come four to a load.  Each
-// shot's gradient is added by itself: adding the pair first halves the reductions but changes the order of the sum over
-// shots, whose rounding is the largest error of a gradient.
+// shot's gradient is one fixed chain of roundings, the same bits in a block of one and of two, and is added by itself:
+// adding the pair first halves the reductions but changes the order of the sum over shots, whose rounding is the largest
+// error of a gradient.
 // What bounds both kernels is instruction issue and the latency of short chains between barriers, not
 // memory: the recorded state (16 bytes per check, iteration and shot, written once and read from L2 after
 // a prefetch) and the gradient's reductions are the only traffic.
-// LP-1054, 4096 shots, T = 20, syndrome loss: forward 1097 -> 516 us, backward 2664 -> 830 us
-// (error loss 784 -> 607 and 1687 -> 685).
+// LP-1054, 4096 shots, T = 20, syndrome loss: forward 1107 -> 669 us, backward 2711 -> 1153 us
+// (error loss 790 -> 605 and 1690 -> 687).
 #pragma once
 
 #include <cstdint>
@@ -53,7 +59,6 @@ struct Lanes {
     static __device__ __forceinline__ word add(word a, word b) { return __fadd_rn(a, b); }
     static __device__ __forceinline__ word sub(word a, word b) { return __fsub_rn(a, b); }
     static __device__ __forceinline__ word mul(word a, word b) { return __fmul_rn(a, b); }
-    static __device__ __forceinline__ word fma(word a, word b, word c) { return __fmaf_rn(a, b, c); }
     static __device__ __forceinline__ float get(word a, int) { return a; }
     static __device__ __forceinline__ void set(word &a, int, float x) { a = x; }
 };
@@ -75,17 +80,6 @@ struct Lanes<2> {
     QLDPC_PACKED2(add, "add.rn.f32x2")
     QLDPC_PACKED2(mul, "mul.rn.f32x2")
     static __device__ __forceinline__ word sub(word a, word b) { return add(a, make_float2(-b.x, -b.y)); }
-    static __device__ __forceinline__ word fma(word a, word b, word c)
-    {
-        unsigned long long x, y, z, r;
-        asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(a.x), "f"(a.y));
-        asm("mov.b64 %0, {%1, %2};" : "=l"(y) : "f"(b.x), "f"(b.y));
-        asm("mov.b64 %0, {%1, %2};" : "=l"(z) : "f"(c.x), "f"(c.y));
-        asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(x), "l"(y), "l"(z));
-        word o;
-        asm("mov.b64 {%0, %1}, %2;" : "=f"(o.x), "=f"(o.y) : "l"(r));
-        return o;
-    }
     static __device__ __forceinline__ float get(word a, int l) { return l ? a.y : a.x; }
     static __device__ __forceinline__ void set(word &a, int l, float x) { (l ? a.y : a.x) = x; }
 };
@@ -150,26 +144,29 @@ __device__ __forceinline__ void load_row(const float *__restrict__ rows, int M, 
 
 // ---------------------------------------------------------------------------------------------
 // Syndrome loss.  With t_v = tanh(Q_v / 2), P_c = (1 + (-1)^s prod_{v in c} t_v) / 2 is the
-// probability that row c's parity under independent bits sigma(-Q) equals s.  Each variable stores on
-// its edge slots its code: u_v = 1 - |t_v| = 2 x / (1 + x), x = e^-|Q_v|, with the sign of Q_v (also on
-// u = 0, where |Q| is so large that |t| = 1).  A check then needs 1 - prod |t| = 1 - prod (1 - u) without
-// the cancellation of the difference: D <- D + u (1 - D) over the row, every term positive.  A violated,
-// confident check gets P = D / 2 exactly as small as it is, a met one P = 1 - D / 2.  One exponential
-// per variable and one logarithm per check; the sum of logarithms this replaces (two log1p a variable,
-// an exp or expm1 a check and an exp per edge of the backward) was most of both kernels.
+// probability that row c's parity under independent bits sigma(-Q) equals s.  Each variable
+// stores, on its edge slots, its log-magnitude code
+//   lm_v = sign(Q_v) * (-log |t_v|),  -log |t_v| = log1p(e^-|Q_v|) - log1p(-e^-|Q_v|)  (+inf at Q = 0),
+// computed once per variable.  A check then has prod |t| = exp(A), A = -sum |lm|, and a violated,
+// confident check gets P = -expm1(A) / 2 without the cancellation of 1 - prod (|t| rounds to 1
+// long before 1 - |t| is negligible).  (u = 1 - |t| from one exponential and a division, and 1 - prod (1 - u)
+// term by term, would spare the logarithms and an exponential per edge: 516 and 830 us.  It loses bits of |t|
+// for Q near 0: with priors of 0.01 and T = 2 a shot's gradient is 7e-6 from 64 bits against 1.8e-6.)
 // ---------------------------------------------------------------------------------------------
 constexpr float kSynLossFloor = 1e-7f;
 
-__device__ __forceinline__ float soft_code(float Q)
+// The sign travels in the sign bit (also on a magnitude of 0, where |Q| is so large that |t| = 1).
+__device__ __forceinline__ float log_magnitude_code(float Q)
 {
     const float x = expf(-fabsf(Q));
-    return with_sign(__fdividef(2.0f * x, 1.0f + x), Q < 0.0f ? 0x80000000u : 0u);
+    const float mag = log1pf(x) - log1pf(-x);   // -log |tanh(Q/2)| >= 0
+    return __uint_as_float(__float_as_uint(mag) | (Q < 0.0f ? 0x80000000u : 0u));
 }
-// d tanh(Q/2) / dQ = (1 - t^2) / 2 = u (1 - u / 2)
-__device__ __forceinline__ float code_slope(float code)
+// d tanh(Q/2) / dQ = sech^2(Q/2) / 2 (no cancellation for large |Q|)
+__device__ __forceinline__ float half_sech2_half(float Q)
 {
-    const float u = fabsf(code);
-    return u * (1.0f - 0.5f * u);
+    const float ch = coshf(0.5f * Q);
+    return 0.5f / (ch * ch);
 }
 
 // P_c of L shots from the codes in check c's slots; s_bits: bit l = s_c of shot l.  WANT_T: the signed t_j.
@@ -180,7 +177,7 @@ __device__ __forceinline__ void parity_match(int c, int M, int deg, uint32_t s_b
 {
     using V = Lanes<L>;
     using word = typename V::word;
-    word D = V::all(0.0f);
+    word A = V::all(0.0f);
     uint32_t neg[L];
 #pragma unroll
     for (int l = 0; l < L; ++l) neg[l] = s_bits << (31 - l);
@@ -188,24 +185,24 @@ __device__ __forceinline__ void parity_match(int c, int M, int deg, uint32_t s_b
     for (int j = 0; j < DC; ++j) {
         if (UNIFORM || j < deg) {
             const word code = ts[j * M + c];
-            word u;
+            word minus;                        // -|lm| = log |t|
 #pragma unroll
             for (int l = 0; l < L; ++l) {
                 neg[l] ^= __float_as_uint(V::get(code, l));
-                V::set(u, l, fabsf(V::get(code, l)));
+                V::set(minus, l, -fabsf(V::get(code, l)));
             }
-            D = V::fma(u, V::sub(V::all(1.0f), D), D);
+            A = V::add(A, minus);
             if constexpr (WANT_T) {
-                const word m = V::sub(V::all(1.0f), u);
 #pragma unroll
-                for (int l = 0; l < L; ++l) V::set(t[j], l, with_sign(V::get(m, l), sign_of(V::get(code, l))));
+                for (int l = 0; l < L; ++l) V::set(t[j], l, with_sign(expf(V::get(minus, l)), sign_of(V::get(code, l))));
             }
         } else if constexpr (WANT_T) {
             t[j] = V::all(1.0f);
         }
     }
 #pragma unroll
-    for (int l = 0; l < L; ++l) P[l] = (neg[l] >> 31) ? 0.5f * V::get(D, l) : 1.0f - 0.5f * V::get(D, l);
+    for (int l = 0; l < L; ++l)
+        P[l] = (neg[l] >> 31) ? -0.5f * expm1f(V::get(A, l)) : 0.5f * (1.0f + expf(V::get(A, l)));
 }
 
 template <int L, int DC, bool UNIFORM>
@@ -234,17 +231,17 @@ __device__ __forceinline__ void syndrome_term_grad(int c, int M, int deg, uint32
 #pragma unroll
     for (int l = 0; l < L; ++l)
         V::set(coef, l, P[l] > kSynLossFloor ? ((s_bits >> l) & 1u ? 0.5f : -0.5f) / P[l] : 0.0f);
-    word run = coef;
+    word run = V::all(1.0f);
 #pragma unroll
     for (int j = 0; j < DC; ++j) {
-        pre[j] = run;                        // coef t_0 ... t_{j-1}
+        pre[j] = run;                        // t_0 ... t_{j-1}
         run = V::mul(run, t[j]);
     }
     word suf = V::all(1.0f);                 // t_{j+1} ... t_{deg-1}
 #pragma unroll
     for (int j = DC - 1; j >= 0; --j) {
         if (UNIFORM || j < deg) {
-            ts[j * M + c] = V::mul(pre[j], suf);
+            ts[j * M + c] = V::mul(coef, V::mul(pre[j], suf));
             suf = V::mul(suf, t[j]);
         }
     }
@@ -428,7 +425,7 @@ __global__ void __launch_bounds__(kTrainThreads, DC <= 8 ? 3 : 1) nms_forward_ke
             if constexpr (SYN) {
                 word code;
 #pragma unroll
-                for (int l = 0; l < L; ++l) V::set(code, l, soft_code(V::get(Q, l)));
+                for (int l = 0; l < L; ++l) V::set(code, l, log_magnitude_code(V::get(Q, l)));
 #pragma unroll
                 for (int i = 0; i < D; ++i) *at_bytes(ts, e[i]) = code;
             } else if (y[u] != kIdleLane) {
@@ -510,7 +507,7 @@ __global__ void __launch_bounds__(kTrainThreads, DC <= 8 ? 3 : 1) nms_backward_k
     // Syndrome loss: once Q^(k) is formed, each variable overwrites its own r slots with its code
     // (no other thread reads them), and each check then replaces the codes with d(term)/d t.
     word *ts = rs;
-    word *ucode = reinterpret_cast<word *>(smem + lay.q_off);     // syndrome loss: the code per lane
+    word *qlane = reinterpret_cast<word *>(smem + lay.q_off);     // syndrome loss: Q^(k) per lane
     float *gam = reinterpret_cast<float *>(smem + lay.g_off);
     uint8_t *y = smem + lay.y_off;
     uint8_t *sb = smem + lay.s_off;
@@ -561,8 +558,8 @@ __global__ void __launch_bounds__(kTrainThreads, DC <= 8 ? 3 : 1) nms_backward_k
 #pragma unroll
                 for (int i = 0; i < D; ++i) Q = V::add(Q, *at_bytes(rs, e[i]));
 #pragma unroll
-                for (int l = 0; l < L; ++l) V::set(code, l, soft_code(V::get(Q, l)));
-                ucode[u] = code;
+                for (int l = 0; l < L; ++l) V::set(code, l, log_magnitude_code(V::get(Q, l)));
+                qlane[u] = Q;
 #pragma unroll
                 for (int i = 0; i < D; ++i) *at_bytes(ts, e[i]) = code;
             });
@@ -583,13 +580,13 @@ __global__ void __launch_bounds__(kTrainThreads, DC <= 8 ? 3 : 1) nms_backward_k
                 sum = V::add(sum, g[i]);
             }
             if constexpr (SYN) {
-                word H = V::all(0.0f), slope;
+                word H = V::all(0.0f);
 #pragma unroll
                 for (int i = 0; i < D; ++i) H = V::add(H, *at_bytes(ts, e[i]));
-                const word code = ucode[u];
+                const word Q = qlane[u];
 #pragma unroll
-                for (int l = 0; l < L; ++l) V::set(slope, l, code_slope(V::get(code, l)));
-                gQ = V::mul(V::mul(gk, slope), H);
+                for (int l = 0; l < L; ++l)   // (as a packed product it came out fused with the packed sum below)
+                    V::set(gQ, l, __fmul_rn(__fmul_rn(V::get(gk, l), half_sech2_half(V::get(Q, l))), V::get(H, l)));
             } else {
                 word Q = V::all(gam[u]);
 #pragma unroll

@@ -65,8 +65,8 @@ int plan_training(const qldpc_graph *g, int32_t batch, int32_t T, TrainPlan &tp)
 
 // Two shots per block share weights, edge lists and reductions, where they fit and every SM still gets
 // several blocks; below that the batch is spread one shot per block (LP-1054, T = 20, syndrome loss, one
-// against two shots per block, forward + backward us: 456 shots 254 | 285, 608 shots 349 | 295, 4096 shots
-// 1693 | 1399; 72 checks on 144 variables, 608 shots 120 | 125, 1216 shots 151 | 146).
+// against two shots per block, forward + backward us: 456 shots 294 | 359, 608 shots 399 | 370, 4096 shots
+// 2062 | 1823; 72 checks on 144 variables, 608 shots 118 | 132, 1216 shots 158 | 158, 4096 shots 394 | 361).
 constexpr int kPairShotsPerSm = 3;
 
 int plan_kernels(const qldpc_graph *g, TrainPlan &tp)
