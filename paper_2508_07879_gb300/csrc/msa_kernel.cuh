@@ -352,6 +352,9 @@ struct RowOut<F32> {
 // r = sign * (w_{m,n} * min_{j != n} |q_j|), w = this iteration's weights in groups of four edges (train_edge_at), read
 // with one 16-byte load a group before the messages, so that their way from L2 overlaps the minima (16384 shots of
 // LP-1054, 20 learned iterations, then the plain ones: 603 us with a 4-byte load where a weight is used -> 549 us).
+// Rows of more than 16 edges read them after the minima, a group at a time: 32 weights beside 32 messages spill (120 rows
+// of 24, two error rates together, us before | after the minima: one shot 276 | 203, 600 shots 971 | 649, 16384 shots
+// 4090 | 3288; rows of 12 lose by it, 16384 shots 1910 | 2036).
 template <class P, int DC, bool UNIFORM, bool LEARNED = false>
 __device__ __forceinline__ int check_step(int c, int M, int deg, uint32_t pw, bool update,
                                           typename P::msg_t *__restrict__ slots, const LaunchParams &p,
@@ -361,8 +364,9 @@ __device__ __forceinline__ int check_step(int c, int M, int deg, uint32_t pw, bo
     using mag_t = typename P::mag_t;
     if (update) {
         acc_t q[DC];
-        float scale[LEARNED ? (DC + 3) / 4 * 4 : 1];
-        if constexpr (LEARNED) {
+        constexpr bool kWeightsFirst = LEARNED && DC <= 16;
+        float scale[kWeightsFirst ? (DC + 3) / 4 * 4 : 1];
+        if constexpr (kWeightsFirst) {
 #pragma unroll
             for (int j = 0; j < DC; j += 4) {
                 float4 v = make_float4(p.alpha, p.alpha, p.alpha, p.alpha);
@@ -381,10 +385,25 @@ __device__ __forceinline__ int check_step(int c, int M, int deg, uint32_t pw, bo
         row_minima<P, DC, UNIFORM>(q, deg, m1, m2, sx);
         const uint32_t negall = ((pw >> 1) ^ (sx >> 31)) & 1u;   // (-1)^{s_m} * prod of all signs
         const RowOut<P> out(m1, m2, negall, p);
+        if constexpr (LEARNED && !kWeightsFirst) {
+            if (w) {
+#pragma unroll
+                for (int j = 0; j < DC; j += 4) {
+                    if (UNIFORM || j < deg) {
+                        const float4 v = __ldg(reinterpret_cast<const float4 *>(w + train_edge_at(4, c, j, M)));
+                        const float x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                        for (int i = 0; i < 4 && j + i < DC; ++i)
+                            if (UNIFORM || j + i < deg) slots[(j + i) * M + c] = out(q[j + i], p, x[i]);
+                    }
+                }
+                return (pw & 1u) == 0;
+            }
+        }
 #pragma unroll
         for (int j = 0; j < DC; ++j) {
             if (UNIFORM || j < deg) {
-                if constexpr (LEARNED)
+                if constexpr (kWeightsFirst)
                     slots[j * M + c] = out(q[j], p, scale[j]);
                 else
                     slots[j * M + c] = typename P::msg_t(out(q[j], p));
