@@ -609,12 +609,24 @@ int occupancy_grid(const qldpc_graph *g0, const void *k, int threads, size_t sme
 //
 // Chosen automatically while it has the shorter time: its threads hold the graph in registers and so issue the
 // fewest instructions per iteration, but its large blocks leave an SM idle at their barriers.  With three
-// or more blocks on an SM they cover for each other and it wins at any batch; with two or one, only up to 48 and
-// 24 shots per SM.  Measured (us, single-shot kernel | best other kernel and block size), FP32 / INT16:
-//   144 x 288, 4 and 3 blocks:  65536 shots 690 | 772 / 794 | 878
-//   192 x 400, 2 blocks:        6400 shots 338 | 351 / 373 | 391;   16384 shots 794 | 755 / 883 | 830
-//   465 x 1054, 1 block:        3200 shots 176 | 184 / 210 | 207;   6400 shots 287 | 261 / 345 | 303
-int64_t latency_limit(int per_sm) { return per_sm >= 3 ? INT64_MAX : per_sm == 2 ? 48 : 24; }
+// or more blocks on an SM they cover for each other and it wins at any batch; with two only up to 48 shots per SM;
+// with one up to 16, in fixed point and with learned weights 12.  Those are rows of one degree of 6 to 9.  Rows of
+// other degrees go through masked loops of up to 8, 16 or 32 edges, whose registers leave fewer blocks an SM and
+// whose length all threads of a block wait for: up to 16 edges it wins up to 4 shots per SM (2 in fixed point), up to 8
+// edges with three blocks an SM at any batch (40), above 16 edges not at all.  Measured (us over error rates 0.01, 0.03
+// and 0.05 together, single-shot kernel | best other kernel), FP32 / INT8:
+//   192 x 400, rows of 7, 2 blocks:   40 shots per SM 501 | 524 / 552 | 580;   64 738 | 731 / 816 | 812
+//   465 x 1054, rows of 8, 1 block:   12 shots per SM 357 | 354 / 417 | 404;   24 608 | 544 / 712 | 602
+//   300 x 600, rows of 6, 1 block:    16 shots per SM 169 | 192 / 220 | 200;   32 246 | 245 / 358 | 281
+//   240 x 720, rows of 12:             4 shots per SM 227 | 242 / 287 | 237;   16 549 | 446 / 730 | 429
+//   120 x 720, rows of 24:             2 shots per SM 437 | 288 / 543 | 230;   16 1888 | 761 / 2419 | 642
+int64_t latency_limit(const KernelChoice &kc, int precision, int per_sm)
+{
+    const bool fixed = precision != QLDPC_FP32;
+    if (kc.uniform) return per_sm >= 3 ? INT64_MAX : per_sm == 2 ? 48 : fixed || kc.learned ? 12 : 16;
+    if (kc.dc > 16) return 1;
+    return kc.dc == 8 && per_sm >= 3 ? (fixed ? 40 : INT64_MAX) : fixed ? 2 : 4;
+}
 
 int plan_latency(const qldpc_graph *const *gs, int nprob, int32_t batch, int precision, bool learned, Plan &pl,
                  bool &chosen)
@@ -649,7 +661,7 @@ int plan_latency(const qldpc_graph *const *gs, int nprob, int32_t batch, int pre
     } else if (int64_t(batch) * nprob > g0->sm_count) {   // (else every shot gets its own SM)
         int per_sm = 0;
         if (int rc = blocks_per_sm(k, threads, smem, per_sm)) return rc;
-        if (per_sm < 1 || shots_per_sm(g0, nprob, batch) > latency_limit(per_sm)) return QLDPC_OK;
+        if (per_sm < 1 || shots_per_sm(g0, nprob, batch) > latency_limit(pl.kc, precision, per_sm)) return QLDPC_OK;
         if (int rc = occupancy_grid(g0, k, threads, smem, nprob, batch, per_sm, pl.grid)) return rc;
     }
     chosen = true;
@@ -665,8 +677,19 @@ int plan_latency(const qldpc_graph *const *gs, int nprob, int32_t batch, int pre
 // 20000 shots 3268 | 3454 and 2355 | 2705, 49152 shots 7330 | 7326 and 5141 | 5223, 65536 shots 9618 | 9499 and 6697 |
 // 6668; at the ends 16384 shots at 0.01 248 | 291 and 157 | 258, 65536 shots at 0.05 3838 | 3617 and 2565 | 2398).
 // INT16 and INT8: where the noisiest decodes cross, 80 and 40 shots per SM (LP-1054 at 0.05: INT16 12000 shots 956 |
-// 938, 16384 shots 1258 | 1182; INT8 8192 shots 662 | 588).
-//
+// 938, 16384 shots 1258 | 1182; INT8 8192 shots 662 | 588): a pair's word of two integers costs the arithmetic of one
+// shot, so noisy batches gain more than quiet ones lose, where FP32 pairs do two shots' arithmetic.
+// Rows of other degrees than 6 to 9 (us at 0.01, 0.03 and 0.05 together, one shot | two): the longer the row, the later
+// FP32 gains (rows of 12, 160 shots per SM 2570 | 2400; rows of 24, 320 shots per SM 8400 | 11000) and the sooner fixed
+// point does: INT16 past 24 shots per SM, above 16 edges past 80 (rows of 12, 32 shots per SM 820 | 745; rows of 24 64
+// 2380 | 2310), INT8 past 2, above 16 edges always (rows of 12, 8 shots per SM 331 | 324; rows of 24 2 327 | 230).
+int64_t pair_line(const KernelChoice &kc, int precision)
+{
+    if (kc.uniform) return precision == QLDPC_INT8 ? 40 : precision == QLDPC_INT16 ? 80 : 320;
+    if (precision == QLDPC_FP32) return kc.dc > 16 ? INT64_MAX : 320;
+    return precision == QLDPC_INT16 ? (kc.dc > 16 ? 80 : 24) : kc.dc > 16 ? 1 : 2;
+}
+
 // Threads per block.  Barriers and uneven last passes cost large blocks more than their shots' shorter
 // latency gives while there are shots for many blocks: a quarter of the checks, at most 128 (65536 shots
 // in pairs, us at 64 / 96 / 128 threads: LP-1054 FP32 2164 / 1798 / 1639, the 192-check code 2477 / 2536 / 2754).  With
@@ -675,14 +698,25 @@ int plan_latency(const qldpc_graph *const *gs, int nprob, int32_t batch, int pre
 // 212, 3200 shots 367 / 383 / 493; the 192-check code learned, 6400 shots at 64 / 128: 319 / 272).  A graph of which
 // few shots fit an SM's shared memory gets the threads that fill it, 1024 an SM (640 in pairs, whose threads need
 // more registers): 1800 checks, 4096 shots at 128 / 256 / 512 threads 716 / 507 / 440.
-int batch_threads(const qldpc_graph *const *gs, int nprob, int64_t per_sm, size_t smem, bool packed)
+// Rows of other degrees than 6 to 9 keep 256 threads up to 24 shots per SM and 128 past them, pairs 128 throughout (a
+// check takes longer, so fewer checks a thread; and a graph of few long rows has more variables than checks to walk:
+// 120 rows of 24 on 720 variables in INT16 pairs, 80 shots per SM at 32 / 128 threads 4610 / 2740; 240 rows of 12 FP32, 24
+// shots per SM at 128 / 256 590 / 580, 80 at 64 / 128 1500 / 1390).  Where few of their pairs fit an SM, 256: 600 rows of
+// 20, INT8, 40 shots per SM at 128 / 160 / 256 2364 / 2550 / 1958.
+int batch_threads(const KernelChoice &kc, const qldpc_graph *const *gs, int nprob, int64_t per_sm, size_t smem)
 {
     int m = 1;
     for (int i = 0; i < nprob; ++i) m = std::max(m, int(gs[i]->m));
-    const int by_shots = per_sm <= 4 ? 512 : per_sm <= 12 ? 256 : per_sm <= 64 ? 128 : std::min(128, round32((m + 3) / 4));
+    int by_shots;
+    if (kc.uniform)
+        by_shots = per_sm <= 4 ? 512 : per_sm <= 12 ? 256 : per_sm <= 64 ? 128 : std::min(128, round32((m + 3) / 4));
+    else
+        by_shots = kc.packed ? 128 : per_sm <= 4 ? 512 : per_sm <= 24 ? 256 : 128;
     const int resident = int(std::max<size_t>(1, (gs[0]->smem_optin + 1024) / (smem + 1024)));   // blocks by shared memory
-    const int fill = (packed ? 640 : 1024) / resident / 32 * 32;
-    return std::min({packed ? kPackedMaxThreads : 1024, round32(m), std::max(by_shots, fill)});
+    int fill = (kc.packed ? 640 : 1024) / resident / 32 * 32;
+    if (kc.packed && !kc.uniform && fill > 128) fill = 256;
+    const int rows = kc.packed && !kc.uniform && per_sm <= 64 ? std::max(128, round32(m)) : round32(m);
+    return std::min({kc.packed ? kPackedMaxThreads : 1024, rows, std::max(by_shots, fill)});
 }
 
 int plan_batch(const qldpc_graph *const *gs, int nprob, int32_t batch, int precision, bool learned, Plan &pl)
@@ -697,8 +731,9 @@ int plan_batch(const qldpc_graph *const *gs, int nprob, int32_t batch, int preci
             if (forced) return QLDPC_ERR_UNSUPPORTED;
             packed = false;
         }
+    pl.kc = variant(gs, nprob, false, learned);
     if (packed && !forced) {
-        packed = per_sm > (precision == QLDPC_INT8 ? 40 : precision == QLDPC_INT16 ? 80 : 320);
+        packed = per_sm > pair_line(pl.kc, precision);
         // and only where two shots fit a block's shared memory (beside 1 KB of static shared
         // memory); a graph whose single shot just fits keeps one shot per block
         for (int i = 0; i < nprob; ++i)
@@ -708,9 +743,8 @@ int plan_batch(const qldpc_graph *const *gs, int nprob, int32_t batch, int preci
     for (int i = 0; i < nprob; ++i)
         smem = std::max(smem, packed ? packed_layout(gs[i]->m, gs[i]->nv, gs[i]->dc_max, word).total
                                      : shot_smem(gs[i], precision));
-    pl.kc = variant(gs, nprob, false, learned);
     pl.kc.packed = packed;
-    pl.threads = g0->user_threads ? g0->user_threads : batch_threads(gs, nprob, per_sm, smem, packed);
+    pl.threads = g0->user_threads ? g0->user_threads : batch_threads(pl.kc, gs, nprob, per_sm, smem);
     if (packed && pl.threads > kPackedMaxThreads) return QLDPC_ERR_UNSUPPORTED;
     pl.smem = smem;
     const void *k = msa_kernel(precision, pl.kc);
