@@ -140,14 +140,16 @@ using I8 = IFix<int8_t, 2, 127>;
 
 // The same arithmetic with 4-byte slots.  The variable lanes are packed so that a warp's slots fall in distinct
 // 4-byte banks; 2- and 1-byte slots share banks (1.5 wavefronts an access on LP-1054) and need conversions.  The
-// single-shot kernel, whose shared memory is never short, keeps its messages so.
-template <class P>
+// single-shot kernel, whose shared memory is never short, keeps its messages so.  Not INT8 rows of more than 16 edges:
+// a check's loads then leave no time to its barriers, and bytes take a quarter of the wavefronts (120 rows of 24 at error
+// rate 0.05, one shot 150 us with 4-byte slots, 131 with bytes; INT16 152 and 154).
+template <class P, int DC>
 struct WideSlots {
     using type = P;
 };
-template <class MSG, int FRAC, int LIM>
-struct WideSlots<IFix<MSG, FRAC, LIM>> {
-    using type = IFix<int32_t, FRAC, LIM>;
+template <class MSG, int FRAC, int LIM, int DC>
+struct WideSlots<IFix<MSG, FRAC, LIM>, DC> {
+    using type = IFix<typename std::conditional<sizeof(MSG) == 1 && (DC > 16), MSG, int32_t>::type, FRAC, LIM>;
 };
 
 template <class T>
@@ -845,12 +847,11 @@ __global__ void __launch_bounds__(kLatencyMaxThreads, 1) msa_latency_kernel(cons
 template <class P, bool LEARNED = false>
 const void *kernel_table(const KernelChoice &kc)
 {
-    using W = typename kern::WideSlots<P>::type;   // (the single-shot kernel's slots: latency_layout with 4 bytes)
 #define QLDPC_K(DCV, UNI, DVV)                                                                  \
     if (kc.dc == DCV && kc.uniform == UNI && kc.dvb == DVV)                                     \
         return !kc.latency      ? reinterpret_cast<const void *>(&kern::msa_batch_kernel<P, DCV, UNI, DVV, LEARNED>) \
-               : kc.one_pass    ? reinterpret_cast<const void *>(&kern::msa_latency_kernel<W, DCV, UNI, DVV, 1, LEARNED>) \
-                                : reinterpret_cast<const void *>(&kern::msa_latency_kernel<W, DCV, UNI, DVV, 2, LEARNED>);
+               : kc.one_pass    ? reinterpret_cast<const void *>(&kern::msa_latency_kernel<typename kern::WideSlots<P, DCV>::type, DCV, UNI, DVV, 1, LEARNED>) \
+                                : reinterpret_cast<const void *>(&kern::msa_latency_kernel<typename kern::WideSlots<P, DCV>::type, DCV, UNI, DVV, 2, LEARNED>);
     QLDPC_VARIANTS(QLDPC_K)
 #undef QLDPC_K
     return nullptr;

@@ -157,7 +157,7 @@ struct KernelChoice {
 constexpr int kLatencyCnPerThread = 2;
 constexpr int kLatencyVnPerThread = 2;
 constexpr int kLatencyMaxThreads = 640;
-constexpr int kLatencySlotBytes = 4;   // in every precision (WideSlots)
+constexpr int kLatencySlotBytes = 4;   // at most, in every precision (WideSlots)
 
 // ---------------------------------------------------------------------------------------------
 // Persistent server (server_kernel.cuh): worker blocks that take requests of any code from one
