@@ -767,13 +767,20 @@ int plan_layered(const qldpc_graph *const *gs, int nprob, int32_t batch, int pre
     pl.kc = variant(gs, nprob, false, false);
     pl.kc.layered = true;
     pl.threads = std::min(1024, round32(widest));
-    // Up to 40 shots per SM (80 in blocks of two warps, of which an SM holds more), with at most 8 layers of rows of degree <= 8 and at most 256 checks per layer: the
+    // With at most 8 layers of rows of degree <= 8 and at most 256 checks per layer, up to some shots per SM: the
     // register-resident kernel (each thread owns one check per layer; Q is the only shared array) has the shorter
-    // time.  Larger batches take the shared-memory kernel, whose smaller register footprint keeps more shots per SM.
-    // FP32, register | shared-memory (us): LP-1054 304 shots 55 | 66, 3200 shots 157 | 173, 6400 shots 213 | 210, 65536
-    // shots 1491 | 911; the 192-check code in layer order (64 threads) 1000 shots 127 | 160, 6400 shots 268 | 314, 16384 shots
-    // 567 | 588, 65536 1997 | 1831.
-    bool reg = pl.threads <= 256 && shots_per_sm(g0, nprob, batch) <= (pl.threads <= 64 ? 80 : 40);
+    // time.  Larger batches take the shared-memory kernel, whose smaller register footprint keeps more shots per SM; the
+    // line lies where the times at error rates 0.01, 0.03 and 0.05 together cross, later in blocks of two warps, of which an
+    // SM holds more, and in fixed point, whose conversions the shared-memory kernel repeats at every access.  Register |
+    // shared-memory (us):
+    //   LP-1054, 96 threads: FP32 304 shots (at 0.03) 55 | 66, 20 shots per SM 484 | 465, 40 717 | 607; INT16 20 524 | 553, 30
+    //   653 | 627; INT8 20 532 | 568, 30 663 | 648
+    //   the 192-check code in layer order, 64 threads: FP32 60 shots per SM 1266 | 1300, 80 1602 | 1600, 100 1938 | 1897; INT16
+    //   80 1740 | 1796, 100 2104 | 2127, 120 2475 | 2454; INT8 80 1793 | 1836, 100 2171 | 2168
+    //   (codes of 72 and 144 checks, 32 and 64 threads: they cross at 150 and 55 in FP32, past 200 in fixed point, within 7 % all the way)
+    const bool fixed = precision != QLDPC_FP32;
+    const int line = pl.threads <= 64 ? (fixed ? 100 : 80) : fixed ? 24 : 16;
+    bool reg = pl.threads <= 256 && shots_per_sm(g0, nprob, batch) <= line;
     for (int i = 0; i < nprob; ++i) reg = reg && gs[i]->dg.nlayers <= 8 && gs[i]->dc_max <= 8 && gs[i]->n <= 65536;
     pl.kc.dvb = reg ? 1 : 0;
     if (reg) {

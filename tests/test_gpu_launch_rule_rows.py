@@ -86,3 +86,25 @@ def test_no_far_slower_kernel(code, mode, per_sm):
         g.set_launch(kernel)
         took[kernel] = microseconds(lambda: q.decode(g, s, prior, **how))
     assert took["auto"] <= 1.5 * min(took.values()), took
+
+
+@pytest.mark.parametrize("mode", ["fp32", "int16", "int8"])
+@pytest.mark.parametrize("code", ["lp1054", "hgp400"])
+def test_layered_lines(code, mode):
+    """Register-resident up to the line, shared-memory past it: the same results, and no batch at a line that takes longer
+    than one just past it (at 40 shots per SM on LP-1054, where the line lay once, a fifth longer in FP32)."""
+    from paper_2508_07879_gb300 import qldpc as q
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    h = (w.lp_code(1054) if code == "lp1054" else w.hgp_code(400)).hz_csr
+    h = w.csr_rows(h, w.layer_order(h)) if code == "hgp400" else h
+    g = q.Graph.from_csr(h)
+    lines = (16, 24, 40) if code == "lp1054" else (80, 100)
+    s = torch.from_numpy(w.syndromes(h, w.iid_x_errors(h.n, 0.05, (lines[-1] + 1) * sms, seed=13))).cuda()
+    prior = torch.full((h.n,), w.prior_llr(0.05), device="cuda")
+    how = dict(max_iter=30, alpha=0.75, precision=mode, layered=True, want_post=True)
+    for per_sm in lines:
+        n, more = per_sm * sms, per_sm * sms + sms
+        past = q.decode(g, s[:more], prior, **how)
+        assert all(torch.equal(a, b[:n]) for a, b in zip(q.decode(g, s[:n], prior, **how), past))
+        at, over = (microseconds(lambda: q.decode(g, s[:k], prior, **how)) for k in (n, more))
+        assert at <= 1.12 * over, (per_sm, at, over)
