@@ -501,12 +501,14 @@ size_t shot_smem(const qldpc_graph *g, int precision)
     return smem_layout(g->m, g->nv, g->dc_max, msg_bytes(precision)).total;
 }
 
-// Opt in to more than 48 KB of dynamic shared memory once per kernel variant and size.
+// Opt in to more than 48 KB of dynamic shared memory once per device, kernel variant and size (the attribute belongs
+// to the kernel on the current device).
 // The kernel's own static shared memory counts against the same per-block limit, so a launch
 // whose dynamic part fits only without it is refused here (UNSUPPORTED) rather than failing.
 int ensure_kernel_attrs(const void *k, size_t smem, size_t smem_optin)
 {
     struct Entry {
+        int device;
         const void *k;
         size_t static_bytes, granted;
     };
@@ -514,15 +516,17 @@ int ensure_kernel_attrs(const void *k, size_t smem, size_t smem_optin)
     static std::vector<Entry> known;
     if (!k) return QLDPC_ERR_UNSUPPORTED;
     if (smem > smem_optin) return QLDPC_ERR_UNSUPPORTED;
+    int dev = 0;
+    if (cudaError_t e = cudaGetDevice(&dev)) return cuda_status(e);
     std::lock_guard<std::mutex> lk(mu);
     Entry *en = nullptr;
     for (auto &x : known)
-        if (x.k == k) en = &x;
+        if (x.device == dev && x.k == k) en = &x;
     if (!en) {
         cudaFuncAttributes fa{};
         cudaError_t e = cudaFuncGetAttributes(&fa, k);
         if (e != cudaSuccess) return cuda_status(e);
-        known.push_back(Entry{k, fa.sharedSizeBytes, 0});
+        known.push_back(Entry{dev, k, fa.sharedSizeBytes, 0});
         en = &known.back();
     }
     if (smem + en->static_bytes > smem_optin) return QLDPC_ERR_UNSUPPORTED;
