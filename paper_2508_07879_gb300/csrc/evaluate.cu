@@ -420,7 +420,7 @@ cudaError_t launch_sample(const DeviceGraph &g, uint64_t seed, int64_t first_sho
                           double p_hi, uint8_t *err, uint8_t *syn, int sm_count, cudaStream_t stream)
 {
     const int64_t tiles = (int64_t(batch) + kern::kSampleShots - 1) / kern::kSampleShots;
-    if (2 * tiles <= sm_count && g.n <= 48 * 1024 - 64)
+    if (2 * tiles <= sm_count)   // (a graph that fits on chip has fewer than 48 K variables)
         kern::sample_shot_kernel<<<std::min(batch, sm_count * 8), kern::kSampleThreads, size_t(g.n), stream>>>(
             g, seed, first_shot, batch, p_lo, p_hi - p_lo, err, syn);
     else   // a block a tile: the last wave fills best

@@ -69,27 +69,8 @@ struct F32 {
         asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
         return r;
     }
-    static __device__ __forceinline__ mag_t scale(mag_t m, const LaunchParams &p)
-    {
-        return __fmul_rn(p.alpha, m);
-    }
     // bit 31 = [x < 0] (valid because no message is -0)
     static __device__ __forceinline__ uint32_t sign_word(acc_t x) { return __float_as_uint(x); }
-    // sign * m with sign = (-1)^{negall} * sign(x): the sign bit flipped, one logic operation
-    // (-m is exact, also -0 for m = 0 as in the oracle)
-    static __device__ __forceinline__ acc_t signed_like(mag_t m, acc_t x, uint32_t negall)
-    {
-        return __uint_as_float(__float_as_uint(m) ^ (__float_as_uint(x) & 0x80000000u) ^ (negall << 31));
-    }
-    // the same in two steps: the check's factor on a magnitude once, then each edge's own sign
-    static __device__ __forceinline__ mag_t presign(mag_t m, uint32_t negall)
-    {
-        return __uint_as_float(__float_as_uint(m) ^ (negall << 31));
-    }
-    static __device__ __forceinline__ acc_t apply_sign(mag_t pm, acc_t x)
-    {
-        return __uint_as_float(__float_as_uint(pm) ^ (__float_as_uint(x) & 0x80000000u));
-    }
     static __device__ __forceinline__ float post(acc_t a) { return a; }
     static __device__ __forceinline__ msg_t to_msg(acc_t q) { return q; }
 };
@@ -125,11 +106,8 @@ struct IFix {
         return (m * p.alpha_q) >> 15;
     }
     static __device__ __forceinline__ uint32_t sign_word(acc_t x) { return uint32_t(x); }
-    static __device__ __forceinline__ acc_t signed_like(mag_t m, acc_t x, uint32_t negall)
-    {
-        const int32_t neg = int32_t(negall ^ (uint32_t(x) >> 31));   // 0 or 1
-        return (m ^ -neg) + neg;
-    }
+    // sign * m with sign = (-1)^{negall} * sign(x), in two steps: the check's factor on a magnitude once, then each edge's
+    // own sign
     static __device__ __forceinline__ mag_t presign(mag_t m, uint32_t negall) { return negall ? -m : m; }
     static __device__ __forceinline__ acc_t apply_sign(mag_t pm, acc_t x) { return x < 0 ? -pm : pm; }
     static __device__ __forceinline__ float post(acc_t a) { return float(a) * (1.0f / float(1 << FRAC)); }

@@ -34,7 +34,7 @@ struct DeviceGraph {
     const int32_t *layer_ptr;// [nlayers + 1] layered schedule: checks of layer l are
     const uint32_t *layer_chk;//   layer_chk[layer_ptr[l] .. layer_ptr[l+1]) (ascending)
     const uint16_t *layer_col;// [m * layer_width] variables of the check at each place of layer_chk, rows padded to
-    int32_t layer_width;     //   whole 16-byte groups (nullptr when an index exceeds 65535)
+    int32_t layer_width;     //   whole 16-byte groups
     int32_t nlayers, max_layer;
     int32_t m, n, nnz;
     int32_t nv;              // variable lanes (n <= nv)

@@ -277,7 +277,7 @@ struct HostLayout {
     std::vector<uint32_t> ecol;    // [dc_max * m] caller's variable of each slot, ~0 for padding
     std::vector<int32_t> layer_ptr;// [nlayers + 1] layered schedule
     std::vector<uint32_t> layer_chk;// [m] checks ordered by (layer, index)
-    std::vector<uint16_t> layer_col;// [m * layer_width] their variables (empty when n > 65535)
+    std::vector<uint16_t> layer_col;// [m * layer_width] their variables
     int32_t layer_width = 0;
     int32_t max_layer = 0;
     int32_t nv = 0;               // variable lanes (n + idle lanes)
@@ -464,13 +464,12 @@ int validate_and_layout(const int32_t *row_ptr, const int32_t *col_idx, int32_t 
     std::vector<int32_t> fillp(out.layer_ptr.begin(), out.layer_ptr.end() - 1);
     for (int32_t i = 0; i < m; ++i) out.layer_chk[size_t(fillp[size_t(layer[size_t(i)])]++)] = uint32_t(i);
     out.layer_width = (dc_max + 7) / 8 * 8;
-    if (n <= 65535) {
-        out.layer_col.assign(size_t(m) * size_t(out.layer_width), uint16_t(0));
-        for (int32_t x = 0; x < m; ++x) {
-            const int32_t i = int32_t(out.layer_chk[size_t(x)]);
-            for (int32_t e = row_ptr[i]; e < row_ptr[i + 1]; ++e)
-                out.layer_col[size_t(x) * out.layer_width + size_t(e - row_ptr[i])] = uint16_t(col_idx[e]);
-        }
+    // (16 bits hold the variables of every graph that fits on chip: 8 bytes a variable allow some 29000)
+    out.layer_col.assign(size_t(m) * size_t(out.layer_width), uint16_t(0));
+    for (int32_t x = 0; x < m; ++x) {
+        const int32_t i = int32_t(out.layer_chk[size_t(x)]);
+        for (int32_t e = row_ptr[i]; e < row_ptr[i + 1]; ++e)
+            out.layer_col[size_t(x) * out.layer_width + size_t(e - row_ptr[i])] = uint16_t(col_idx[e]);
     }
     return QLDPC_OK;
 }
@@ -790,9 +789,6 @@ int plan_layered(const qldpc_graph *const *gs, int nprob, int32_t batch, int pre
     if (reg) {
         smem = 0;
         for (int i = 0; i < nprob; ++i) smem = std::max(smem, align16(size_t(gs[i]->n) * 4));
-    } else {
-        for (int i = 0; i < nprob; ++i)   // (a shot of so many variables does not fit either)
-            if (!gs[i]->dg.layer_col) return QLDPC_ERR_UNSUPPORTED;
     }
     pl.smem = smem;
     const void *k = msa_kernel(precision, pl.kc);
@@ -1093,7 +1089,7 @@ int qldpc_graph_create(const int32_t *row_ptr, const int32_t *col_idx, int32_t m
     g->dg.vslot16 = hl.vslot16.empty() ? nullptr : reinterpret_cast<const uint16_t *>(b + offs[10]);
     g->dg.vlane = reinterpret_cast<const uint32_t *>(b + offs[11]);
     g->dg.vchk16 = hl.vchk16.empty() ? nullptr : reinterpret_cast<const uint16_t *>(b + offs[12]);
-    g->dg.layer_col = hl.layer_col.empty() ? nullptr : reinterpret_cast<const uint16_t *>(b + offs[13]);
+    g->dg.layer_col = reinterpret_cast<const uint16_t *>(b + offs[13]);
     g->dg.layer_width = hl.layer_width;
     g->dg.ncls = int32_t(hl.cls_end.size());
     for (size_t c = 0; c < hl.cls_end.size(); ++c) {
