@@ -87,6 +87,20 @@ NCU_TRAFFIC = {"msa_batch_kernel": {"source": "msa_kernel.cuh", "source_sha16": 
                "msa_packed_kernel": {"source": "msa_packed.cuh", "source_sha16": "7e5f890b9cc2f38f",
                                      "bytes_per_launch": 39615684}}
 
+# The library's own choice of kernel for LP-1054 (one single-shot block an SM) by shots per SM: the single-shot kernel up to
+# the first, one shot per block up to the second, two past it.
+KERNEL_LINES = {"fp32": (16, 320), "int16": (12, 80), "int8": (12, 40)}
+
+
+def kernel_label(kernel: str, batch: int, sms: int, precision: str) -> str:
+    """Name of the kernel that decodes a batch of LP-1054 under a launch setting."""
+    single, one = KERNEL_LINES[precision]
+    per_sm = -(-batch // sms)
+    if kernel == "auto":
+        kernel = "latency" if per_sm <= single else "batch" if per_sm <= one else "packed"
+    return f"msa_{kernel}_kernel"
+
+
 FALLBACK_HBM_GBS = 6800.0     # the profiling recipe's fallback when MEASURED_PEAKS.json is absent
 WORKLOAD = "LP-1054 H_Z (465x1054, E=3720), iid X noise p=0.01..0.05, B=65536/step, max 50 it, alpha 0.75"
 
@@ -453,7 +467,7 @@ def run_ours(args, rank, world, local):
     # edge-iterations it runs: E x (iterations summed over its 65536 shots)
     props = torch.cuda.get_device_properties(dev)
     clocks = clk.summary(lo, hi)
-    kernel_name = "msa_batch_kernel" if args.kernel == "batch" else "msa_packed_kernel"
+    kernel_name = kernel_label(args.kernel, B, props.multi_processor_count, args.precision)
     roofline = decoder_roofline(h, B, iters_per_batch, args.steps, ms_per_step, args.precision,
                                 props.multi_processor_count, clocks["sm_max_mhz"] or 2070.0, kernel_name)
 
@@ -1051,10 +1065,14 @@ def measure_serving(qldpc, args, learned_weights=None):
 def measure_precisions(qldpc, graph, syn_d, pri_d, out, stream, B, args, steps=100):
     """Flooding decode of the benchmark's batches in each precision: throughput and decoded fraction."""
     import torch
+    sms = torch.cuda.get_device_properties(syn_d[0].device).multi_processor_count
+    shots = {"latency": "one shot per block, graph in registers", "batch": "one shot per block", "packed": "two shots per block"}
     res = {}
     for name in ("fp32", "int16", "int8", "fp32_one_shot", "int16_one_shot", "int8_one_shot"):
         prec = name.split("_")[0]
-        graph.set_launch("batch" if name.endswith("_one_shot") else "auto")
+        kernel = "batch" if name.endswith("_one_shot") else "auto"
+        graph.set_launch(kernel)
+        label = kernel_label(kernel, B, sms, prec)
         ok = iters = 0
         with torch.cuda.stream(stream):
             for j in range(len(syn_d)):
@@ -1076,8 +1094,7 @@ def measure_precisions(qldpc, graph, syn_d, pri_d, out, stream, B, args, steps=1
             stream.synchronize()
         res[name] = {"value": B * steps / (e0.elapsed_time(e1) / 1e3), "unit": "syndromes/s",
                      "decoded_fraction": ok / (len(syn_d) * B), "mean_iters": iters / (len(syn_d) * B),
-                     "kernel": "msa_batch_kernel (one shot per block)" if name.endswith("_one_shot")
-                     else "msa_packed_kernel (two shots per block)"}
+                     "kernel": f"{label} ({shots[label.split('_')[1]]})"}
     graph.set_launch("auto")
     return res
 
