@@ -681,14 +681,18 @@ int plan_latency(const qldpc_graph *const *gs, int nprob, int32_t batch, int pre
 // 6668; at the ends 16384 shots at 0.01 248 | 291 and 157 | 258, 65536 shots at 0.05 3838 | 3617 and 2565 | 2398).
 // INT16 and INT8: where the noisiest decodes cross, 80 and 40 shots per SM (LP-1054 at 0.05: INT16 12000 shots 956 |
 // 938, 16384 shots 1258 | 1182; INT8 8192 shots 662 | 588): a pair's word of two integers costs the arithmetic of one
-// shot, so noisy batches gain more than quiet ones lose, where FP32 pairs do two shots' arithmetic.
+// shot, so noisy batches gain more than quiet ones lose, where FP32 pairs do two shots' arithmetic.  Codes of at most 256
+// checks, whose blocks of one shot have 64 threads (batch_threads) and so are twice as many, gain later: INT16 past 240 and
+// INT8 past 90 (the 192-check code, us at 0.01, 0.03 and 0.05 together: INT16 160 shots per SM 1659 | 1736, 320 3042 | 2975;
+// INT8 80 926 | 960, 108 1171 | 1127; INT16 108 at 0.01 156 | 246).
 // Rows of other degrees than 6 to 9 (us at 0.01, 0.03 and 0.05 together, one shot | two): the longer the row, the later
 // FP32 gains (rows of 12, 160 shots per SM 2570 | 2400; rows of 24, 320 shots per SM 8400 | 11000) and the sooner fixed
 // point does: INT16 past 24 shots per SM, above 16 edges past 80 (rows of 12, 32 shots per SM 820 | 745; rows of 24 64
 // 2380 | 2310), INT8 past 2, above 16 edges always (rows of 12, 8 shots per SM 331 | 324; rows of 24 2 327 | 230).
-int64_t pair_line(const KernelChoice &kc, int precision)
+int64_t pair_line(const KernelChoice &kc, int precision, int m)
 {
-    if (kc.uniform) return precision == QLDPC_INT8 ? 40 : precision == QLDPC_INT16 ? 80 : 320;
+    if (kc.uniform && precision == QLDPC_FP32) return 320;
+    if (kc.uniform) return precision == QLDPC_INT16 ? (m <= 256 ? 240 : 80) : m <= 256 ? 90 : 40;
     if (precision == QLDPC_FP32) return kc.dc > 16 ? INT64_MAX : 320;
     return precision == QLDPC_INT16 ? (kc.dc > 16 ? 80 : 24) : kc.dc > 16 ? 1 : 2;
 }
@@ -736,7 +740,9 @@ int plan_batch(const qldpc_graph *const *gs, int nprob, int32_t batch, int preci
         }
     pl.kc = variant(gs, nprob, false, learned);
     if (packed && !forced) {
-        packed = per_sm > pair_line(pl.kc, precision);
+        int m = 1;
+        for (int i = 0; i < nprob; ++i) m = std::max(m, int(gs[i]->m));
+        packed = per_sm > pair_line(pl.kc, precision, m);
         // and only where two shots fit a block's shared memory (beside 1 KB of static shared
         // memory); a graph whose single shot just fits keeps one shot per block
         for (int i = 0; i < nprob; ++i)
