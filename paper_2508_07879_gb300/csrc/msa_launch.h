@@ -336,9 +336,10 @@ struct TrainChoice {
     int dvb;         // column-degree bucket 4/8/16
 };
 
-// Kernels of one (x1) or two (x2) shots per block; nullptr: no such variant.
-const void *train_kernel_x1(const TrainChoice &tc, int loss_kind, bool backward);
-const void *train_kernel_x2(const TrainChoice &tc, int loss_kind, bool backward);
+// Forward kernels of one (x1) or two (x2) shots per block, and the backward kernel; nullptr: no such variant.
+const void *train_forward_x1(const TrainChoice &tc, int loss_kind);
+const void *train_forward_x2(const TrainChoice &tc, int loss_kind);
+const void *train_backward(const TrainChoice &tc, int loss_kind);
 cudaError_t launch_training(const void *kernel, const TrainParams &p, int grid, int threads, size_t smem,
                             cudaStream_t stream);
 cudaError_t launch_permute_weights(const float *w_csr, const DeviceGraph &g, int32_t T, int32_t wstride, int group,

@@ -1,4 +1,4 @@
-// Training of the learned decoder: the one-shot-per-block kernels of nms_train.cuh, the weights' row layout,
+// Training of the learned decoder: the one-shot-per-block kernels of nms_train.cuh, the weights' edge groups,
 // and the Adam step.
 #include <algorithm>
 #include <cmath>
@@ -57,9 +57,19 @@ __global__ void adam_kernel(float *__restrict__ param, const float *__restrict__
 
 }  // namespace kern
 
-const void *train_kernel_x1(const TrainChoice &tc, int loss_kind, bool backward)
+const void *train_forward_x1(const TrainChoice &tc, int loss_kind) { return forward_kernel<1>(tc, loss_kind); }
+
+const void *train_backward(const TrainChoice &tc, int loss_kind)
 {
-    return backward ? train_kernel<1, true>(tc, loss_kind) : train_kernel<1, false>(tc, loss_kind);
+    const bool syn = loss_kind == kLossSyndrome;
+#define QLDPC_K(DCV, UNI, DVV)                                                                  \
+    if (tc.dc == DCV && tc.uniform == UNI && tc.dvb == DVV)                                     \
+        return syn ? reinterpret_cast<const void *>(&kern::nms_backward_kernel<DCV, UNI, DVV, true>) \
+                   : reinterpret_cast<const void *>(&kern::nms_backward_kernel<DCV, UNI, DVV, false>);
+    QLDPC_TRAIN_SHORT(QLDPC_K)
+    QLDPC_TRAIN_LONG(QLDPC_K)
+#undef QLDPC_K
+    return nullptr;
 }
 
 cudaError_t launch_training(const void *kernel, const TrainParams &p, int grid, int threads, size_t smem,

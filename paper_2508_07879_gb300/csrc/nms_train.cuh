@@ -24,18 +24,18 @@
 //                        its 74400 weights then differ in the last bit, and after one more step the two
 //                        gradients are more than 2e-5 apart for 3 of 10 inputs (up to 4e-3).
 //
-// L = 1 or 2 shots per block.  Two shots share every weight, edge list and prior, their messages sit in one
+// Forward, L = 1 or 2 shots per block: two shots share every weight, edge list and prior, their messages sit in one
 // 8-byte slot per edge (as in the two-shots-per-block decoder), their sums and products are packed FP32
 // operations.  Weights and their gradient lie in groups of four edges (two where a row's length asks for it), so a
-// check moves four of them per instruction and a warp whole sectors; a lane's edge slots come four to a load.  Each
-// shot's gradient is one fixed chain of roundings, the same bits in a block of one and of two, and is added by itself:
-// adding the pair first halves the reductions but changes the order of the sum over shots, whose rounding is the largest
-// error of a gradient.
+// check moves four of them per instruction and a warp whole sectors; a lane's edge slots come four to a load.
+// Backward, one shot per block, a few blocks an SM that take the shots in waves: a shot's gradient is one fixed
+// chain of roundings, and the sum over shots, whose rounding is the largest error of a gradient, keeps the order of those
+// waves (plan_backward in qldpc_learned.cpp).
 // What bounds both kernels is instruction issue and the latency of short chains between barriers, not
 // memory: the recorded state (16 bytes per check, iteration and shot, written once and read from L2 after
 // a prefetch) and the gradient's reductions are the only traffic.
-// LP-1054, 4096 shots, T = 20, syndrome loss: forward 1107 -> 669 us, backward 2711 -> 1153 us
-// (error loss 790 -> 605 and 1690 -> 687).
+// LP-1054, 4096 shots, T = 20, syndrome loss: forward 1107 -> 669 us, backward 2711 -> 1572 us
+// (error loss 790 -> 605 and 1690 -> 1038).
 #pragma once
 
 #include <cstdint>
@@ -218,31 +218,24 @@ __device__ __forceinline__ void syndrome_term(int c, int M, int deg, uint32_t s_
 
 // d(syndrome term)/d t_j = -(1 / P) (-1)^s / 2 prod_{i != j} t_i (0 at the floor), written over the
 // codes of check c.
-template <int L, int DC, bool UNIFORM>
-__device__ __forceinline__ void syndrome_term_grad(int c, int M, int deg, uint32_t s_bits,
-                                                   typename Lanes<L>::word *__restrict__ ts)
+template <int DC, bool UNIFORM>
+__device__ __forceinline__ void syndrome_term_grad(int c, int M, int deg, uint32_t s_bit, float *__restrict__ ts)
 {
-    using V = Lanes<L>;
-    using word = typename V::word;
-    float P[L];
-    word t[DC], pre[DC];
-    parity_match<L, DC, UNIFORM, true>(c, M, deg, s_bits, ts, P, t);
-    word coef;
-#pragma unroll
-    for (int l = 0; l < L; ++l)
-        V::set(coef, l, P[l] > kSynLossFloor ? ((s_bits >> l) & 1u ? 0.5f : -0.5f) / P[l] : 0.0f);
-    word run = V::all(1.0f);
+    float P[1], t[DC], pre[DC];
+    parity_match<1, DC, UNIFORM, true>(c, M, deg, s_bit, ts, P, t);
+    const float coef = P[0] > kSynLossFloor ? (s_bit & 1u ? 0.5f : -0.5f) / P[0] : 0.0f;
+    float run = 1.0f;
 #pragma unroll
     for (int j = 0; j < DC; ++j) {
         pre[j] = run;                        // t_0 ... t_{j-1}
-        run = V::mul(run, t[j]);
+        run = __fmul_rn(run, t[j]);
     }
-    word suf = V::all(1.0f);                 // t_{j+1} ... t_{deg-1}
+    float suf = 1.0f;                        // t_{j+1} ... t_{deg-1}
 #pragma unroll
     for (int j = DC - 1; j >= 0; --j) {
         if (UNIFORM || j < deg) {
-            ts[j * M + c] = V::mul(coef, V::mul(pre[j], suf));
-            suf = V::mul(suf, t[j]);
+            ts[j * M + c] = __fmul_rn(coef, __fmul_rn(pre[j], suf));
+            suf = __fmul_rn(suf, t[j]);
         }
     }
 }
@@ -471,229 +464,172 @@ __device__ __forceinline__ void prefetch_state(const uint4 *st, int M, int tid, 
 
 // r of check c recomputed from its recorded state and its edges' weights (bit-identical to the
 // forward's r).
-template <int L, int DC, bool UNIFORM>
-__device__ __forceinline__ void recompute_r(int c, int M, int deg, const uint4 (&st)[L], const float (&w)[DC],
-                                            typename Lanes<L>::word *__restrict__ rs)
+template <int DC, bool UNIFORM>
+__device__ __forceinline__ void recompute_r(int c, int M, int deg, const uint4 &st, const float (&w)[DC], float *__restrict__ rs)
 {
-    using V = Lanes<L>;
-    uint32_t flip[L];
+    const uint32_t flip = st.z ^ (0u - ((st.w >> 16) & 1u));   // bit j: the sign of r_j
 #pragma unroll
-    for (int l = 0; l < L; ++l) flip[l] = st[l].z ^ (0u - ((st[l].w >> 16) & 1u));   // bit j: the sign of r_j
-#pragma unroll
-    for (int j = 0; j < DC; ++j) {
-        if (UNIFORM || j < deg) {
-            typename V::word mu;
-#pragma unroll
-            for (int l = 0; l < L; ++l)
-                V::set(mu, l, with_sign(__uint_as_float(j == int(st[l].w & 0xffu) ? st[l].y : st[l].x),
-                                        (flip[l] << (31 - j)) & 0x80000000u));
-            rs[j * M + c] = V::mul(V::all(w[j]), mu);
-        }
-    }
+    for (int j = 0; j < DC; ++j)
+        if (UNIFORM || j < deg)
+            rs[j * M + c] = __fmul_rn(w[j], with_sign(__uint_as_float(j == int(st.w & 0xffu) ? st.y : st.x),
+                                                      (flip << (31 - j)) & 0x80000000u));
 }
 
-template <int L, int DC, bool UNIFORM, int DV, bool SYN>
-__global__ void __launch_bounds__(kTrainThreads, DC <= 8 ? 3 : 1) nms_backward_kernel(const __grid_constant__ TrainParams p)
+// One shot per block, shots blockIdx.x, blockIdx.x + gridDim.x, ... (plan_backward in qldpc_learned.cpp).
+template <int DC, bool UNIFORM, int DV, bool SYN>
+__global__ void __launch_bounds__(kTrainThreads, DC <= 8 ? 2 : 1) nms_backward_kernel(const __grid_constant__ TrainParams p)
 {
-    using V = Lanes<L>;
-    using word = typename V::word;
     const DeviceGraph &G = p.g;
     const int M = G.m, N = G.n, NV = G.nv, T = blockDim.x, tid = threadIdx.x;
     const size_t S = size_t(M) * p.wstride;
     extern __shared__ __align__(16) unsigned char smem[];
-    const TrainLayout lay = train_layout(M, NV, G.dc_max, L, true, SYN);
-    word *gs = reinterpret_cast<word *>(smem + lay.slot_off);     // dL/dq (next iteration), then dL/dr
-    word *rs = reinterpret_cast<word *>(smem + lay.r_off);        // recomputed r of the current iteration
+    const TrainLayout lay = train_layout(M, NV, G.dc_max, 1, true, SYN);
+    float *gs = reinterpret_cast<float *>(smem + lay.slot_off);   // dL/dq (next iteration), then dL/dr
+    float *rs = reinterpret_cast<float *>(smem + lay.r_off);      // recomputed r of the current iteration
     // Syndrome loss: once Q^(k) is formed, each variable overwrites its own r slots with its code
     // (no other thread reads them), and each check then replaces the codes with d(term)/d t.
-    word *ts = rs;
-    word *qlane = reinterpret_cast<word *>(smem + lay.q_off);     // syndrome loss: Q^(k) per lane
+    float *ts = rs;
+    float *qlane = reinterpret_cast<float *>(smem + lay.q_off);   // syndrome loss: Q^(k) per lane
     float *gam = reinterpret_cast<float *>(smem + lay.g_off);
     uint8_t *y = smem + lay.y_off;
     uint8_t *sb = smem + lay.s_off;
-    int shot[L];
-    bool real[L];
-    block_shots<L>(p.batch, shot, real);
-    const uint4 *st[L];
-    word gscale;
-#pragma unroll
-    for (int l = 0; l < L; ++l) {
-        st[l] = p.state + size_t(shot[l]) * p.T * M;
-        V::set(gscale, l, real[l] ? p.grad_loss[shot[l]] * (1.0f / float(SYN ? M : N)) : 0.0f);
-        if (p.T > 1) prefetch_state(st[l] + size_t(p.T - 2) * M, M, tid, T);
-    }
+    for (int u = tid; u < NV; u += T) gam[u] = F32::quantize(lane_prior(G, p.prior, u));
+    for (int b = blockIdx.x; b < p.batch; b += gridDim.x) {   // (the last iteration's barrier closes a shot)
+        const int shot[1] = {b};
+        const uint4 *st = p.state + size_t(b) * p.T * M;
+        const float gscale = p.grad_loss[b] * (1.0f / float(SYN ? M : N));
+        if (p.T > 1) prefetch_state(st + size_t(p.T - 2) * M, M, tid, T);
 
-    // iteration T: recompute r; dL/dq of iteration T+1 is zero
-    for (int c = tid; c < M; c += T) {
-        const int deg = UNIFORM ? DC : int(__ldg(G.rdeg + c));
-        if (SYN) sb[c] = check_bits<L>(p.syn, shot, M, c);
-        float w[DC];
-        uint4 s[L];
+        // iteration T: recompute r; dL/dq of iteration T+1 is zero
+        for (int c = tid; c < M; c += T) {
+            const int deg = UNIFORM ? DC : int(__ldg(G.rdeg + c));
+            if (SYN) sb[c] = check_bits<1>(p.syn, shot, M, c);
+            float w[DC];
+            const uint4 s = __ldg(st + size_t(p.T - 1) * M + c);
+            load_row<DC, UNIFORM>(p.w + size_t(p.T - 1) * S, M, c, deg, w);
+            recompute_r<DC, UNIFORM>(c, M, deg, s, w, rs);
 #pragma unroll
-        for (int l = 0; l < L; ++l) s[l] = __ldg(st[l] + size_t(p.T - 1) * M + c);
-        load_row<DC, UNIFORM>(p.w + size_t(p.T - 1) * S, M, c, deg, w);
-        recompute_r<L, DC, UNIFORM>(c, M, deg, s, w, rs);
-#pragma unroll
-        for (int j = 0; j < DC; ++j)
-            if (UNIFORM || j < deg) gs[j * M + c] = V::all(0.0f);
-    }
-    for (int u = tid; u < NV; u += T) {
-        gam[u] = F32::quantize(lane_prior(G, p.prior, u));
-        if constexpr (!SYN) y[u] = lane_targets<L>(G, p.target, shot, u);
-    }
-    __syncthreads();
-    for (int k = p.T - 1; k >= 0; --k) {
-        if (k > 1) {
-#pragma unroll
-            for (int l = 0; l < L; ++l) prefetch_state(st[l] + size_t(k - 2) * M, M, tid, T);
+            for (int j = 0; j < DC; ++j)
+                if (UNIFORM || j < deg) gs[j * M + c] = 0.0f;
         }
-        const word gk = V::mul(gscale, V::all(p.loss_w ? __ldg(p.loss_w + k) : 1.0f / float(p.T)));
-        if constexpr (SYN) {
-            // the code of Q^(k) on every edge slot, then each check's d(loss term)/d t in its place
+        if constexpr (!SYN)
+            for (int u = tid; u < NV; u += T) y[u] = lane_targets<1>(G, p.target, shot, u);
+        __syncthreads();
+        for (int k = p.T - 1; k >= 0; --k) {
+            if (k > 1) prefetch_state(st + size_t(k - 2) * M, M, tid, T);
+            const float gk = __fmul_rn(gscale, p.loss_w ? __ldg(p.loss_w + k) : 1.0f / float(p.T));
+            if constexpr (SYN) {
+                // the code of Q^(k) on every edge slot, then each check's d(loss term)/d t in its place
+                for_lanes<DV>(G, tid, T, [&](auto deg, int u) {
+                    constexpr int D = decltype(deg)::value;
+                    uint32_t e[D > 0 ? D : 1];
+                    lane_slots<D, sizeof(float)>(G.vslot16, NV, u, e);
+                    float Q = gam[u];
+#pragma unroll
+                    for (int i = 0; i < D; ++i) Q = __fadd_rn(Q, *at_bytes(rs, e[i]));
+                    const float code = log_magnitude_code(Q);
+                    qlane[u] = Q;
+#pragma unroll
+                    for (int i = 0; i < D; ++i) *at_bytes(ts, e[i]) = code;
+                });
+                __syncthreads();
+                for (int c = tid; c < M; c += T)
+                    syndrome_term_grad<DC, UNIFORM>(c, M, UNIFORM ? DC : int(__ldg(G.rdeg + c)), sb[c], ts);
+                __syncthreads();
+            }
+            // variable side: dL/dQ^(k) (error loss: Q^(k) from the recomputed r), and dL/dr for every edge
             for_lanes<DV>(G, tid, T, [&](auto deg, int u) {
                 constexpr int D = decltype(deg)::value;
                 uint32_t e[D > 0 ? D : 1];
-                lane_slots<D, sizeof(word)>(G.vslot16, NV, u, e);
-                word Q = V::all(gam[u]), code;
+                float g[D > 0 ? D : 1], sum = 0.0f, gQ;
+                lane_slots<D, sizeof(float)>(G.vslot16, NV, u, e);
 #pragma unroll
-                for (int i = 0; i < D; ++i) Q = V::add(Q, *at_bytes(rs, e[i]));
+                for (int i = 0; i < D; ++i) {
+                    g[i] = *at_bytes(gs, e[i]);
+                    sum = __fadd_rn(sum, g[i]);
+                }
+                if constexpr (SYN) {
+                    float H = 0.0f;
 #pragma unroll
-                for (int l = 0; l < L; ++l) V::set(code, l, log_magnitude_code(V::get(Q, l)));
-                qlane[u] = Q;
+                    for (int i = 0; i < D; ++i) H = __fadd_rn(H, *at_bytes(ts, e[i]));
+                    gQ = __fmul_rn(__fmul_rn(gk, half_sech2_half(qlane[u])), H);
+                } else {
+                    float Q = gam[u];
 #pragma unroll
-                for (int i = 0; i < D; ++i) *at_bytes(ts, e[i]) = code;
+                    for (int i = 0; i < D; ++i) Q = __fadd_rn(Q, *at_bytes(rs, e[i]));
+                    gQ = __fmul_rn(gk, float(y[u] & 1u) - sigmoid(-Q));
+                }
+#pragma unroll
+                for (int i = 0; i < D; ++i) *at_bytes(gs, e[i]) = __fadd_rn(gQ, __fsub_rn(sum, g[i]));
             });
             __syncthreads();
-            for (int c = tid; c < M; c += T)
-                syndrome_term_grad<L, DC, UNIFORM>(c, M, UNIFORM ? DC : int(__ldg(G.rdeg + c)), sb[c], ts);
-            __syncthreads();
-        }
-        // variable side: dL/dQ^(k) (error loss: Q^(k) from the recomputed r), and dL/dr for every edge
-        for_lanes<DV>(G, tid, T, [&](auto deg, int u) {
-            constexpr int D = decltype(deg)::value;
-            uint32_t e[D > 0 ? D : 1];
-            word g[D > 0 ? D : 1], sum = V::all(0.0f), gQ;
-            lane_slots<D, sizeof(word)>(G.vslot16, NV, u, e);
+            // check side: weight gradient, dL/dq of iteration k, and r of iteration k-1
+            for (int c = tid; c < M; c += T) {
+                const int deg = UNIFORM ? DC : int(__ldg(G.rdeg + c));
+                constexpr int GW = edge_group<DC, UNIFORM>(), PAD = (DC + GW - 1) / GW * GW;
+                float w[DC], dw[PAD];
+                const uint4 s = __ldg(st + size_t(k) * M + c);
+                load_row<DC, UNIFORM>(p.w + size_t(k) * S, M, c, deg, w);
+                uint4 sp{};
+                if (k > 0) sp = __ldg(st + size_t(k - 1) * M + c);
+                const uint32_t flip = s.z ^ (0u - ((s.w >> 16) & 1u));
+                const int i1 = int(s.w & 0xffu), i2 = int((s.w >> 8) & 0xffu);
+                float rest = 0.0f, own = 0.0f;     // sum of gr w sign over the edges but idx1, and idx1's
 #pragma unroll
-            for (int i = 0; i < D; ++i) {
-                g[i] = *at_bytes(gs, e[i]);
-                sum = V::add(sum, g[i]);
-            }
-            if constexpr (SYN) {
-                word H = V::all(0.0f);
-#pragma unroll
-                for (int i = 0; i < D; ++i) H = V::add(H, *at_bytes(ts, e[i]));
-                const word Q = qlane[u];
-#pragma unroll
-                for (int l = 0; l < L; ++l)   // (as a packed product it came out fused with the packed sum below)
-                    V::set(gQ, l, __fmul_rn(__fmul_rn(V::get(gk, l), half_sech2_half(V::get(Q, l))), V::get(H, l)));
-            } else {
-                word Q = V::all(gam[u]);
-#pragma unroll
-                for (int i = 0; i < D; ++i) Q = V::add(Q, *at_bytes(rs, e[i]));
-#pragma unroll
-                for (int l = 0; l < L; ++l)
-                    V::set(gQ, l, V::get(gk, l) * (float((y[u] >> l) & 1u) - sigmoid(-V::get(Q, l))));
-            }
-#pragma unroll
-            for (int i = 0; i < D; ++i) *at_bytes(gs, e[i]) = V::add(gQ, V::sub(sum, g[i]));
-        });
-        __syncthreads();
-        // check side: weight gradient, dL/dq of iteration k, and r of iteration k-1
-        for (int c = tid; c < M; c += T) {
-            const int deg = UNIFORM ? DC : int(__ldg(G.rdeg + c));
-            constexpr int GW = edge_group<DC, UNIFORM>(), PAD = (DC + GW - 1) / GW * GW;
-            float w[DC], dw[L][PAD];
-            uint4 s[L], sp[L];
-#pragma unroll
-            for (int l = 0; l < L; ++l) s[l] = __ldg(st[l] + size_t(k) * M + c);
-            load_row<DC, UNIFORM>(p.w + size_t(k) * S, M, c, deg, w);
-            if (k > 0) {
-#pragma unroll
-                for (int l = 0; l < L; ++l) sp[l] = __ldg(st[l] + size_t(k - 1) * M + c);
-            }
-            uint32_t flip[L];
-            float rest[L], own[L];     // sum of gr w sign over the edges but idx1, and idx1's
-#pragma unroll
-            for (int l = 0; l < L; ++l) {
-                flip[l] = s[l].z ^ (0u - ((s[l].w >> 16) & 1u));
-                rest[l] = own[l] = 0.0f;
-            }
-#pragma unroll
-            for (int j = 0; j < PAD; ++j) {
-#pragma unroll
-                for (int l = 0; l < L; ++l) dw[l][j] = 0.0f;
-                if (j < DC && (UNIFORM || j < deg)) {
-                    const word gr = gs[j * M + c];
-                    word sg;           // gr * sign
-#pragma unroll
-                    for (int l = 0; l < L; ++l) V::set(sg, l, with_sign(V::get(gr, l), (flip[l] << (31 - j)) & 0x80000000u));
-                    const word t = V::mul(sg, V::all(w[j]));
-#pragma unroll
-                    for (int l = 0; l < L; ++l) {
-                        const bool min1 = j == int(s[l].w & 0xffu);
-                        dw[l][j] = __fmul_rn(V::get(sg, l), __uint_as_float(min1 ? s[l].y : s[l].x));
-                        if (min1)
-                            own[l] = V::get(t, l);
+                for (int j = 0; j < PAD; ++j) {
+                    dw[j] = 0.0f;
+                    if (j < DC && (UNIFORM || j < deg)) {
+                        const float sg = with_sign(gs[j * M + c], (flip << (31 - j)) & 0x80000000u);   // gr * sign
+                        const float t = __fmul_rn(sg, w[j]);
+                        dw[j] = __fmul_rn(sg, __uint_as_float(j == i1 ? s.y : s.x));
+                        if (j == i1)
+                            own = t;
                         else
-                            rest[l] += V::get(t, l);
+                            rest = __fadd_rn(rest, t);
+                        gs[j * M + c] = 0.0f;
                     }
-                    gs[j * M + c] = V::all(0.0f);
                 }
-            }
-            float *out = p.partial + size_t(k) * S;
-#pragma unroll
-            for (int l = 0; l < L; ++l)
+                float *out = p.partial + size_t(k) * S;
 #pragma unroll
                 for (int j = 0; j < PAD; j += GW)     // (results unused: reductions; 0 past the row's end)
-                    if (real[l] && (UNIFORM || j < deg)) {
+                    if (UNIFORM || j < deg) {
                         float *at = out + train_edge_at(GW, c, j, M);
                         if constexpr (GW == 2)
-                            atomicAdd(reinterpret_cast<float2 *>(at), make_float2(dw[l][j], dw[l][j + 1]));
+                            atomicAdd(reinterpret_cast<float2 *>(at), make_float2(dw[j], dw[j + 1]));
                         else
-                            atomicAdd(reinterpret_cast<float4 *>(at),
-                                      make_float4(dw[l][j], dw[l][j + 1], dw[l][j + 2], dw[l][j + 3]));
+                            atomicAdd(reinterpret_cast<float4 *>(at), make_float4(dw[j], dw[j + 1], dw[j + 2], dw[j + 3]));
                     }
-            // dL/dq is 0 but at the positions of the two minima
-            float *g1 = reinterpret_cast<float *>(gs);
-#pragma unroll
-            for (int l = 0; l < L; ++l) {
-                const int i1 = int(s[l].w & 0xffu), i2 = int((s[l].w >> 8) & 0xffu);
-                g1[(i1 * M + c) * L + l] = (s[l].z >> i1) & 1u ? -rest[l] : rest[l];
-                g1[(i2 * M + c) * L + l] = (s[l].z >> i2) & 1u ? -own[l] : own[l];
+                // dL/dq is 0 but at the positions of the two minima
+                gs[i1 * M + c] = (s.z >> i1) & 1u ? -rest : rest;
+                gs[i2 * M + c] = (s.z >> i2) & 1u ? -own : own;
+                if (k > 0) {
+                    load_row<DC, UNIFORM>(p.w + size_t(k - 1) * S, M, c, deg, w);
+                    recompute_r<DC, UNIFORM>(c, M, deg, sp, w, rs);
+                }
             }
-            if (k > 0) {
-                load_row<DC, UNIFORM>(p.w + size_t(k - 1) * S, M, c, deg, w);
-                recompute_r<L, DC, UNIFORM>(c, M, deg, sp, w, rs);
-            }
+            __syncthreads();
         }
-        __syncthreads();
     }
 }
 
 }  // namespace kern
 
 // Compiled training variants: uniform row degree 6..8 with column-degree bucket 4 or 8, or a row-degree
-// bucket 8 with column-degree bucket 8 or 16 (both for one and two shots per block); longer rows take one
+// bucket 8 with column-degree bucket 8 or 16 (forward: for one and two shots per block); longer rows take one
 // shot per block.
 #define QLDPC_TRAIN_SHORT(X)                                                                    \
     X(6, true, 4) X(6, true, 8) X(7, true, 4) X(7, true, 8) X(8, true, 4) X(8, true, 8)        \
     X(8, false, 8) X(8, false, 16)
 #define QLDPC_TRAIN_LONG(X) X(16, false, 8) X(16, false, 16) X(32, false, 8) X(32, false, 16)
 
-template <int L, bool BACKWARD>
-const void *train_kernel(const TrainChoice &tc, int loss_kind)
+template <int L>
+const void *forward_kernel(const TrainChoice &tc, int loss_kind)
 {
     const bool syn = loss_kind == kLossSyndrome;
 #define QLDPC_K(DCV, UNI, DVV)                                                                  \
-    if (tc.dc == DCV && tc.uniform == UNI && tc.dvb == DVV) {                                   \
-        if constexpr (BACKWARD)                                                                 \
-            return syn ? reinterpret_cast<const void *>(&kern::nms_backward_kernel<L, DCV, UNI, DVV, true>) \
-                       : reinterpret_cast<const void *>(&kern::nms_backward_kernel<L, DCV, UNI, DVV, false>); \
-        else                                                                                    \
-            return syn ? reinterpret_cast<const void *>(&kern::nms_forward_kernel<L, DCV, UNI, DVV, true>) \
-                       : reinterpret_cast<const void *>(&kern::nms_forward_kernel<L, DCV, UNI, DVV, false>); \
-    }
+    if (tc.dc == DCV && tc.uniform == UNI && tc.dvb == DVV)                                     \
+        return syn ? reinterpret_cast<const void *>(&kern::nms_forward_kernel<L, DCV, UNI, DVV, true>) \
+                   : reinterpret_cast<const void *>(&kern::nms_forward_kernel<L, DCV, UNI, DVV, false>);
     QLDPC_TRAIN_SHORT(QLDPC_K)
     if constexpr (L == 1) {
         QLDPC_TRAIN_LONG(QLDPC_K)

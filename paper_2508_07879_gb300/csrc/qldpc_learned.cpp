@@ -36,8 +36,10 @@ TrainChoice train_choice(const qldpc_graph *g)
 
 struct TrainPlan {
     TrainChoice tc{};
-    int shots = 1, threads = 0, grid = 0;            // per block; blocks
-    const void *kernel[2][2] = {};                   // [loss kind][backward]
+    int shots = 1;                                   // per forward block
+    int threads[2] = {};                             // [backward]
+    int grid[2][2] = {};                             // [loss kind][backward]
+    const void *kernel[2][2] = {};
     size_t smem[2][2] = {};
     int32_t wstride = 0, group = 4;
     size_t w_off = 0, state_off = 0, part_off = 0, total = 0;
@@ -63,21 +65,51 @@ int plan_training(const qldpc_graph *g, int32_t batch, int32_t T, TrainPlan &tp)
     return QLDPC_OK;
 }
 
-// Two shots per block share weights, edge lists and reductions, where they fit and every SM still gets
+// Forward.  Two shots per block share weights and edge lists, where they fit and every SM still gets
 // several blocks; below that the batch is spread one shot per block (LP-1054, T = 20, syndrome loss, one
-// against two shots per block, forward + backward us: 456 shots 294 | 359, 608 shots 399 | 370, 4096 shots
-// 2062 | 1823; 72 checks on 144 variables, 608 shots 118 | 132, 1216 shots 158 | 158, 4096 shots 394 | 361).
+// against two shots per block, us: 456 shots 112 | 133, 608 shots 139 | 135, 4096 shots 725 | 669; 72 checks on 144
+// variables, 608 shots 47 | 51, 1216 shots 62 | 59, 4096 shots 149 | 133).
 constexpr int kPairShotsPerSm = 3;
 
-int plan_kernels(const qldpc_graph *g, TrainPlan &tp)
+int plan_forward(const qldpc_graph *g, int32_t batch, int shots, TrainPlan &tp)
 {
-    for (int kind = 0; kind < 2; ++kind)
-        for (int back = 0; back < 2; ++back) {
-            tp.kernel[kind][back] = tp.shots == 2 ? train_kernel_x2(tp.tc, kind, back) : train_kernel_x1(tp.tc, kind, back);
-            if (!tp.kernel[kind][back]) return QLDPC_ERR_UNSUPPORTED;
-            tp.smem[kind][back] = train_layout(g->m, g->nv, g->dc_max, tp.shots, back, kind == kLossSyndrome).total;
-            if (int rc = ensure_kernel_attrs(tp.kernel[kind][back], tp.smem[kind][back], g->smem_optin)) return rc;
-        }
+    for (int kind = 0; kind < 2; ++kind) {
+        tp.kernel[kind][0] = shots == 2 ? train_forward_x2(tp.tc, kind) : train_forward_x1(tp.tc, kind);
+        if (!tp.kernel[kind][0]) return QLDPC_ERR_UNSUPPORTED;
+        tp.smem[kind][0] = train_layout(g->m, g->nv, g->dc_max, shots, false, kind == kLossSyndrome).total;
+        if (int rc = ensure_kernel_attrs(tp.kernel[kind][0], tp.smem[kind][0], g->smem_optin)) return rc;
+        tp.grid[kind][0] = int((int64_t(batch) + shots - 1) / shots);
+    }
+    tp.shots = shots;
+    // threads: one pass over the checks of a small code
+    tp.threads[0] = std::min(kTrainThreads, std::max(64, (g->m + 31) / 32 * 32));
+    return QLDPC_OK;
+}
+
+// Backward.  One shot per block of 128 threads, four blocks an SM that take the shots in waves (up to two shots per SM, where
+// no order is left to keep, each its own block of the forward's size: LP-1054, 304 shots 149 us).  The blocks add into one
+// buffer, small shares into sums that have grown large, so the order in which shots arrive shows.  LP-1054, 4096 shots,
+// T = 20, syndrome loss: a gradient is off an exactly rounded sum by 7e-6 of its norm, two runs of these waves differ by
+// 5e-7, and other schedules lie further from them than that: two shots per block 7.7e-7 (1153 us, where the waves take
+// 1572), blocks of 192 threads 1.5e-6, the two halves of the batch in turn 5e-6.  What the next step can make of such
+// distances (nms_train.cuh) decides for the order that training has always had.
+constexpr int kBackwardThreads = 128, kBackwardBlocksPerSm = 4, kBackwardWideShotsPerSm = 2;
+
+int plan_backward(const qldpc_graph *g, int32_t batch, TrainPlan &tp)
+{
+    const bool wide = int64_t(batch) <= int64_t(kBackwardWideShotsPerSm) * g->sm_count;
+    tp.threads[1] = wide ? tp.threads[0] : kBackwardThreads;
+    for (int kind = 0; kind < 2; ++kind) {
+        tp.kernel[kind][1] = train_backward(tp.tc, kind);
+        if (!tp.kernel[kind][1]) return QLDPC_ERR_UNSUPPORTED;
+        tp.smem[kind][1] = train_layout(g->m, g->nv, g->dc_max, 1, true, kind == kLossSyndrome).total;
+        if (int rc = ensure_kernel_attrs(tp.kernel[kind][1], tp.smem[kind][1], g->smem_optin)) return rc;
+        int per_sm = 0;
+        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tp.kernel[kind][1], tp.threads[1], tp.smem[kind][1]);
+        if (e != cudaSuccess) return cuda_status(e);
+        if (per_sm < 1) return QLDPC_ERR_UNSUPPORTED;
+        tp.grid[kind][1] = wide ? batch : int(std::min<int64_t>(batch, int64_t(std::min(per_sm, kBackwardBlocksPerSm)) * g->sm_count));
+    }
     return QLDPC_OK;
 }
 
@@ -86,16 +118,11 @@ int plan_training_uncached(const qldpc_graph *g, int32_t batch, int32_t T, Train
     tp.tc = train_choice(g);
     if (tp.tc.dc < 0) return QLDPC_ERR_UNSUPPORTED;
     if (!g->dg.vslot16) return QLDPC_ERR_UNSUPPORTED;   // (more edge slots than any training block holds)
-    tp.shots = int64_t(batch) > int64_t(kPairShotsPerSm) * g->sm_count ? 2 : 1;
-    int rc = plan_kernels(g, tp);
-    if (rc == QLDPC_ERR_UNSUPPORTED && tp.shots == 2) {
-        tp.shots = 1;
-        rc = plan_kernels(g, tp);
-    }
+    int rc = QLDPC_ERR_UNSUPPORTED;
+    if (int64_t(batch) > int64_t(kPairShotsPerSm) * g->sm_count) rc = plan_forward(g, batch, 2, tp);
+    if (rc == QLDPC_ERR_UNSUPPORTED) rc = plan_forward(g, batch, 1, tp);
+    if (!rc) rc = plan_backward(g, batch, tp);
     if (rc) return rc;
-    // threads: one pass over the checks of a small code
-    tp.threads = std::min(kTrainThreads, std::max(64, (g->m + 31) / 32 * 32));
-    tp.grid = int((int64_t(batch) + tp.shots - 1) / tp.shots);
     tp.group = train_group(tp.tc.dc, tp.tc.uniform);
     tp.wstride = (g->dc_max + tp.group - 1) / tp.group * tp.group;
     const size_t rows = size_t(T) * size_t(g->m) * size_t(tp.wstride) * sizeof(float);
@@ -206,7 +233,7 @@ int qldpc_nms_forward(const qldpc_graph *g, const uint8_t *syndromes, const uint
     p.loss_w = loss_weights;
     p.loss_kind = loss;
     cudaError_t e = launch_permute_weights(weights, g->dg, T, tp.wstride, tp.group, const_cast<float *>(p.w), st);
-    if (e == cudaSuccess) e = launch_training(tp.kernel[loss][0], p, tp.grid, tp.threads, tp.smem[loss][0], st);
+    if (e == cudaSuccess) e = launch_training(tp.kernel[loss][0], p, tp.grid[loss][0], tp.threads[0], tp.smem[loss][0], st);
     return cuda_status(e);
 }
 
@@ -229,7 +256,7 @@ int qldpc_nms_backward(const qldpc_graph *g, const uint8_t *syndromes, const uin
     p.loss_w = loss_weights;
     p.loss_kind = loss;
     cudaError_t e = cudaMemsetAsync(p.partial, 0, tp.total - tp.part_off, st);
-    if (e == cudaSuccess) e = launch_training(tp.kernel[loss][1], p, tp.grid, tp.threads, tp.smem[loss][1], st);
+    if (e == cudaSuccess) e = launch_training(tp.kernel[loss][1], p, tp.grid[loss][1], tp.threads[1], tp.smem[loss][1], st);
     if (e == cudaSuccess) e = launch_gather_grad(p.partial, g->dg, T, tp.wstride, tp.group, out_grad, st);
     return cuda_status(e);
 }

@@ -1,5 +1,5 @@
 """A shot's weight gradient to the last bit.  The sum over shots has no fixed order, but a shot's own gradient is one
-chain of operations: the same bits in a block of one shot and of two, the bits of the release before the two-shot blocks
+chain of operations: the same bits alone and in every batch, the bits of the release before two shots per block
 (tests/golden/nms_grad_crc.txt), and an error against 64 bits that the exponential of a code explains.  Last bits matter here:
 a minimum that changes place after the next step moves the whole gradient."""
 import os
