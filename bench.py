@@ -82,10 +82,8 @@ SMEM_BYTES_PER_CLK_PER_SM = 128  # 32 banks x 4 B
 # DRAM bytes of one decoder launch on the benchmark batch (FP32), from ncu captures (the sum of
 # dram__bytes_read.sum and dram__bytes_write.sum, mean over launches of the five rates), valid only for
 # the kernel source they were taken on (sha256 prefix of that file); null once that source changes.
-NCU_TRAFFIC = {"msa_batch_kernel": {"source": "msa_kernel.cuh", "source_sha16": "61e9fb1b9d8386fc",
-                                    "bytes_per_launch": 39156923},
-               "msa_packed_kernel": {"source": "msa_packed.cuh", "source_sha16": "7e5f890b9cc2f38f",
-                                     "bytes_per_launch": 39615684}}
+NCU_TRAFFIC = {"msa_packed_kernel": {"source": "msa_packed.cuh", "source_sha16": "04a32043ab0dbbfc",
+                                     "bytes_per_launch": 40019200}}
 
 # The library's own choice of kernel for LP-1054 (one single-shot block an SM) by shots per SM: the single-shot kernel up to
 # the first, one shot per block up to the second, two past it.

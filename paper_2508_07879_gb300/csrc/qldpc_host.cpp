@@ -686,9 +686,9 @@ int plan_latency(const qldpc_graph *const *gs, int nprob, int32_t batch, int pre
 // INT8 past 90 (the 192-check code, us at 0.01, 0.03 and 0.05 together: INT16 160 shots per SM 1659 | 1736, 320 3042 | 2975;
 // INT8 80 926 | 960, 108 1171 | 1127; INT16 108 at 0.01 156 | 246).
 // Rows of other degrees than 6 to 9 (us at 0.01, 0.03 and 0.05 together, one shot | two): the longer the row, the later
-// FP32 gains (rows of 12, 160 shots per SM 2570 | 2400; rows of 24, 320 shots per SM 8400 | 11000) and the sooner fixed
+// FP32 gains (rows of 12, 160 shots per SM 2570 | 2400; rows of 24, 320 shots per SM 8400 | 10850) and the sooner fixed
 // point does: INT16 past 24 shots per SM, above 16 edges past 80 (rows of 12, 32 shots per SM 820 | 745; rows of 24 64
-// 2380 | 2310), INT8 past 2, above 16 edges always (rows of 12, 8 shots per SM 331 | 324; rows of 24 2 327 | 230).
+// 2380 | 2310), INT8 past 2, above 16 edges always (rows of 12, 8 shots per SM 331 | 324; rows of 24 2 327 | 261).
 int64_t pair_line(const KernelChoice &kc, int precision, int m)
 {
     if (kc.uniform && precision == QLDPC_FP32) return 320;
@@ -782,8 +782,8 @@ int plan_layered(const qldpc_graph *const *gs, int nprob, int32_t batch, int pre
     // line lies where the times at error rates 0.01, 0.03 and 0.05 together cross, later in blocks of two warps, of which an
     // SM holds more, and in fixed point, whose conversions the shared-memory kernel repeats at every access.  Register |
     // shared-memory (us):
-    //   LP-1054, 96 threads: FP32 304 shots (at 0.03) 55 | 66, 20 shots per SM 484 | 465, 40 717 | 607; INT16 20 524 | 553, 30
-    //   653 | 627; INT8 20 532 | 568, 30 663 | 648
+    //   LP-1054, 96 threads: FP32 16 shots per SM 413 | 421, 20 474 | 474, 40 717 | 607; INT16 24 553 | 577, 30
+    //   653 | 627; INT8 24 561 | 585, 30 663 | 648
     //   the 192-check code in layer order, 64 threads: FP32 60 shots per SM 1266 | 1300, 80 1602 | 1600, 100 1938 | 1897; INT16
     //   80 1740 | 1796, 100 2104 | 2127, 120 2475 | 2454; INT8 80 1793 | 1836, 100 2171 | 2168
     //   (codes of 72 and 144 checks, 32 and 64 threads: they cross at 150 and 55 in FP32, past 200 in fixed point, within 7 % all the way)

@@ -36,7 +36,6 @@ TrainChoice train_choice(const qldpc_graph *g)
 
 struct TrainPlan {
     TrainChoice tc{};
-    int shots = 1;                                   // per forward block
     int threads[2] = {};                             // [backward]
     int grid[2][2] = {};                             // [loss kind][backward]
     const void *kernel[2][2] = {};
@@ -80,7 +79,6 @@ int plan_forward(const qldpc_graph *g, int32_t batch, int shots, TrainPlan &tp)
         if (int rc = ensure_kernel_attrs(tp.kernel[kind][0], tp.smem[kind][0], g->smem_optin)) return rc;
         tp.grid[kind][0] = int((int64_t(batch) + shots - 1) / shots);
     }
-    tp.shots = shots;
     // threads: one pass over the checks of a small code
     tp.threads[0] = std::min(kTrainThreads, std::max(64, (g->m + 31) / 32 * 32));
     return QLDPC_OK;
